@@ -177,7 +177,8 @@ typedef struct riot_ctx riot_ctx;
  * observations and the B descriptor to the device, builds L, and allocates
  * all workspace for kmax sketch columns (through opt->dev_alloc when given;
  * a NULL from it is RIOT_ENOMEM, a pointer not aligned to 256 bytes
- * RIOT_EINVAL).  It also looks up, once per device, the device address of
+ * RIOT_EINVAL; only the Lorenz-96 workspace that lets FP64 integrations of a
+ * few columns spread over the GPU may be refused: they then run slower).  It also looks up, once per device, the device address of
  * the static scratch array of riot_hessian_apply_noalloc.  cuda_stream is a
  * cudaStream_t (NULL = legacy default stream).  On failure *out is NULL. */
 riot_status riot_setup(riot_ctx **out, const riot_model_desc *model, const riot_obs_desc *obs,

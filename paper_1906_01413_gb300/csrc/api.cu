@@ -252,6 +252,17 @@ void ev_mark(riot_ctx *c, int phase)
     }
 }
 
+// FP64 Lorenz-96 integrations in the modes of l96_hvp_launch_f64: one or a few columns with
+// their states split over the SMs, more with a column per CTA; r as there.
+cudaError_t l96_f64(riot_ctx *ctx, const double *W, double *Y, int64_t ld, int ncols, int add_identity, double *r,
+                    int mode)
+{
+    int P = 0;
+    if ((mode == 0 || ncols == 1) && l96_split_better(ctx->m, ncols, hvp_f64_plan(ctx->m.geom, ncols, &P)))
+        return l96_split_f64(ctx->m, ctx->coef64, W, Y, ld, ncols, add_identity, r, mode, ctx->s);
+    return l96_hvp_launch_f64(ctx->m, ctx->coef64, W, Y, ld, ncols, add_identity, r, mode, ctx->s);
+}
+
 riot_status hvp(riot_ctx *ctx, const void *W, void *Y, int64_t ld, int ncols, int add_identity)
 {
     if (ctx->model == RIOT_MODEL_ADVDIFF) {
@@ -264,8 +275,7 @@ riot_status hvp(riot_ctx *ctx, const void *W, void *Y, int64_t ld, int ncols, in
         const char *w = (const char *)W + (size_t)c0 * ld * rs;
         char *yv = (char *)Y + (size_t)c0 * ld * rs;
         if (ctx->prec == RIOT_PREC_FP64)
-            CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, (const double *)w, (double *)yv, ld, nc, add_identity,
-                                  (double *)ctx->rscr, 0, ctx->s));
+            CU(l96_f64(ctx, (const double *)w, (double *)yv, ld, nc, add_identity, (double *)ctx->rscr, 0));
         else if (ctx->coefw && (ctx->hvp_kernel == RIOT_HVP_WARP_PAIRS || ctx->hvp_kernel == RIOT_HVP_WARP_SHUFFLE))
             CU(l96_hvp_warp_launch(ctx->m, ctx->coefw, (const float *)w, (float *)yv, ld, nc, add_identity,
                                    (float *)ctx->rscr, ctx->errflag, ctx->s, ctx->hvp_S, ctx->wait_polls,
@@ -282,7 +292,7 @@ riot_status hvp(riot_ctx *ctx, const void *W, void *Y, int64_t ld, int ncols, in
 cudaError_t bsqrt(riot_ctx *ctx, const double *in, double *out, int transpose, int ncols)
 {
     if (ctx->model == RIOT_MODEL_ADVDIFF) return adv_bsqrt(ctx->a, in, out, ncols, ctx->s);   // L symmetric
-    return bsqrt_launch(ctx->m, in, out, transpose, ncols, ctx->s);
+    return bsqrt_launch(ctx->m, in, ctx->n, out, ctx->n, transpose, ncols, nullptr, ctx->s);
 }
 
 // Q (FP64, n x k) = orthonormal basis of Y (real, n x k): shifted CholeskyQR
@@ -491,6 +501,56 @@ void sym_sqrt_host(std::vector<double> &A, int n)
         }
 }
 
+// Tables of the split FP64 integrations and, when memory allows, their workspace: room for a
+// few columns (rows of the observed steps and two states each, 256 MB at most beyond
+// two).  Without it (the allocator returned NULL) those integrations take one CTA a column.
+riot_status setup_split(riot_ctx *ctx, const std::vector<int> &optr, const std::vector<int> &oidx,
+                        const std::vector<double> &rinv)
+{
+    L96Dev &m = ctx->m;
+    const int n = ctx->n, p = ctx->p, T = m.T;
+    std::vector<int> orow(T + 1, -1), rowstep, obsrow(p);
+    for (int t = 0; t <= T; ++t)
+        if (optr[t] < optr[t + 1]) {
+            orow[t] = (int)rowstep.size();
+            rowstep.push_back(t);
+            for (int j = optr[t]; j < optr[t + 1]; ++j) obsrow[j] = orow[t];
+        }
+    const size_t nrow = rowstep.size(), np = (size_t)n, col = (nrow + 2) * np;
+    m.sp.nrow = (int)nrow;
+    m.sp.last_step = nrow ? rowstep.back() : -1;
+    int *d_rowstep = nullptr, *d_obsrow = nullptr;
+    TRY(dalloc(ctx, &d_rowstep, nrow));
+    TRY(dalloc(ctx, &d_obsrow, (size_t)p));
+    m.sp.orow_h = orow;
+    m.sp.rowstep = d_rowstep;
+    m.sp.obsrow = d_obsrow;
+    size_t cols = ((size_t)256 << 20) / (col * sizeof(double));
+    cols = cols > 16 ? 16 : cols;
+    if (cols > (size_t)ctx->kmax) cols = (size_t)ctx->kmax;
+    if (cols < 2) cols = 2;   // the gradient and the product that scales the FP32 path
+    double *wgt = nullptr, *work = nullptr;
+    riot_status st = dalloc(ctx, &wgt, nrow * np);
+    if (st == RIOT_OK) st = dalloc(ctx, &work, cols * col);
+    if (st != RIOT_OK && st != RIOT_ENOMEM) return st;
+    std::vector<double> w;
+    cudaError_t e = cudaSuccess;
+    if (st == RIOT_OK) {
+        w.assign(nrow * np, 0.0);
+        for (int j = 0; j < p; ++j) w[(size_t)obsrow[j] * np + oidx[j]] += rinv[j];
+        e = up(ctx, wgt, w.data(), w.size());
+        m.sp.wgt = wgt;
+        m.sp.rows = work;
+        m.sp.a = work + cols * nrow * np;
+        m.sp.b = m.sp.a + cols * np;
+        m.sp.cols = (int)cols;
+    }
+    if (e || (e = up(ctx, d_rowstep, rowstep.data(), nrow)) ||
+        (e = up(ctx, d_obsrow, obsrow.data(), obsrow.size())) || (e = cudaStreamSynchronize(ctx->s)))
+        return fail(ctx, RIOT_ECUDA, "setup upload failed: %s", cudaGetErrorString(e));
+    return RIOT_OK;
+}
+
 riot_status setup_l96(riot_ctx *ctx, const riot_model_desc *model, const riot_obs_desc *obs, const riot_bcov_desc *B)
 {
     const int64_t n64 = model->n;
@@ -562,6 +622,9 @@ riot_status setup_l96(riot_ctx *ctx, const riot_model_desc *model, const riot_ob
         (e = up(ctx, ctx->sig64, sig.data(), sig.size())) || (e = up(ctx, ctx->sig32, sig32.data(), sig32.size())) ||
         (e = cudaStreamSynchronize(ctx->s)))
         return fail(ctx, RIOT_ECUDA, "setup upload failed: %s", cudaGetErrorString(e));
+    // the padding slots of short chunks stay 0: the trajectory writes its variables only
+    if ((e = cudaMemsetAsync(ctx->coef64, 0, sizeof(double2) * ((size_t)T * 4 * m.geom.Np + 1), ctx->s)))
+        return fail(ctx, RIOT_ECUDA, "setup failed: %s", cudaGetErrorString(e));
     m.optr = ctx->optr;
     m.oslot = ctx->oslot;
     m.oidx = ctx->oidx;
@@ -572,6 +635,7 @@ riot_status setup_l96(riot_ctx *ctx, const riot_model_desc *model, const riot_ob
     m.band32 = ctx->band32;
     m.sig64 = ctx->sig64;
     m.sig32 = ctx->sig32;
+    TRY(setup_split(ctx, optr, oidx, rinv));
     if (ctx->prec == RIOT_PREC_MIXED && warp_kernel_fits(m.geom)) {
         // tables of the warp-synchronous FP32 Hessian kernel
         std::vector<int> ostep, ostart, sslot, perm;
@@ -796,12 +860,16 @@ riot_status setup_common(riot_ctx *ctx)
 // Gaussian w (FP64 product) bounds the leading eigenvalue from below by a
 // factor of order sqrt(n); the exponent keeps sqrt(n) * 16 * that ratio under
 // 2^96, well inside the FP32 range, and is 0 for windows that need none.
+// The caller has put w into ctx->tmp (scale_probe) and A w into ctx->dv.
+cudaError_t scale_probe(riot_ctx *ctx)
+{
+    return normal_launch(ctx->seed ^ 0x9e3779b97f4a7c15ULL, 0x5ca1eu, ctx->n, 1, ctx->n, 1, ctx->tmp, ctx->s);
+}
+
 riot_status choose_scale(riot_ctx *ctx)
 {
     const int n = ctx->n;
     cudaStream_t s = ctx->s;
-    CU(normal_launch(ctx->seed ^ 0x9e3779b97f4a7c15ULL, 0x5ca1eu, n, 1, n, 1, ctx->tmp, s));
-    CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, ctx->tmp, ctx->dv, n, 1, 0, ctx->rd, 0, s));
     CU(cudaMemsetAsync(ctx->nrm, 0, 4 * sizeof(double), s));
     CU(add_half_sq(n, ctx->tmp, ctx->nrm, s));
     CU(add_half_sq(n, ctx->dv, ctx->nrm + 1, s));
@@ -1410,12 +1478,22 @@ riot_status riot_outer_begin(riot_ctx *ctx, const double *x_dev, const double *v
     if (ctx->model == RIOT_MODEL_ADVDIFF) {
         CU(adv_outer(ctx->a, ctx->x, ctx->d, ctx->jo, ctx->rd, ctx->g, ctx->s));
     } else {
-        CU(l96_nl_launch(ctx->m, ctx->x, ctx->traj, ctx->coef32, ctx->coef64, ctx->d, ctx->jo, nullptr, ctx->s));
+        CU(l96_nl_launch(ctx->m, ctx->x, ctx->traj, ctx->coef64, nullptr, ctx->s));
+        if (ctx->coef32) CU(l96_coef32(ctx->m, ctx->coef64, ctx->coef32, ctx->s));
         if (ctx->coefw) CU(l96_coef_warp(ctx->m, ctx->coef64, ctx->coefw, ctx->s));
-        // gradient b = L^T H^T R^-1 d: one FP64 adjoint integration, then g = b + v
-        CU(mul(ctx->p, ctx->d, ctx->rinv64, ctx->rd, ctx->s));
-        CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, nullptr, ctx->g, n, 1, 0, ctx->rd, 1, ctx->s));
-        if (ctx->prec == RIOT_PREC_MIXED) TRY(choose_scale(ctx));
+        // gradient b = L^T H^T R^-1 d by an FP64 adjoint integration, g = b + v below; on the mixed
+        // path also the product of choose_scale, whose adjoint shares that integration
+        const bool split = ctx->m.sp.cols > 0, mixed = ctx->prec == RIOT_PREC_MIXED;
+        CU(l96_innov(ctx->m, ctx->traj, ctx->d, ctx->jo, split, ctx->s));
+        if (mixed) CU(scale_probe(ctx));
+        if (split) {
+            CU(l96_split_gradient(ctx->m, ctx->coef64, ctx->g, mixed ? ctx->tmp : nullptr, ctx->dv, ctx->s));
+        } else {
+            CU(mul(ctx->p, ctx->d, ctx->rinv64, ctx->rd, ctx->s));
+            CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, nullptr, ctx->g, n, 1, 0, ctx->rd, 1, ctx->s));
+            if (mixed) CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, ctx->tmp, ctx->dv, n, 1, 0, ctx->rd, 0, ctx->s));
+        }
+        if (mixed) TRY(choose_scale(ctx));
     }
     CU(axpby(n, 1.0, ctx->v, 1.0, ctx->g, ctx->s));
     // preconditioned loop: the gradient of the problem in w (v = v_{k-1} + P_k w) is P_k^T (b + v)
@@ -1482,8 +1560,7 @@ riot_status riot_hessian_apply_noalloc(riot_ctx *ctx, const void *W_dev, void *Y
         if (ctx->model == RIOT_MODEL_ADVDIFF)
             CU(adv_hvp(ctx->a, ctx->prec == RIOT_PREC_FP64, w, yv, ld, nc, add_identity, scr, ctx->s));
         else if (ctx->prec == RIOT_PREC_FP64)
-            CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, (const double *)w, (double *)yv, ld, nc, add_identity,
-                                  (double *)scr, 0, ctx->s));
+            CU(l96_f64(ctx, (const double *)w, (double *)yv, ld, nc, add_identity, (double *)scr, 0));
         else {
             const int ai = ctx->scale_exp ? 0 : add_identity;
             if (ctx->coefw && (ctx->hvp_kernel == RIOT_HVP_WARP_PAIRS || ctx->hvp_kernel == RIOT_HVP_WARP_SHUFFLE))
@@ -1726,7 +1803,7 @@ riot_status riot_quadratic_cost(riot_ctx *ctx, const double *dv_dev, double *J_o
         // r = R^-1 H M L dv: one FP64 tangent-linear integration along the stored trajectory
         r = ctx->rd;
         if (ctx->model == RIOT_MODEL_ADVDIFF) CU(adv_tl_obs(ctx->a, dv_dev, r, s));
-        else CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, dv_dev, nullptr, n, 1, 0, r, 2, s));
+        else CU(l96_f64(ctx, dv_dev, nullptr, n, 1, 0, r, 2));
     }
     CU(cudaMemsetAsync(ctx->nrm + 2, 0, sizeof(double), s));
     CU(obs_quad_cost(ctx->p, ctx->d, r, ctx->rinv64, ctx->nrm + 2, s));
@@ -1857,8 +1934,8 @@ riot_status riot_l96_forecast(int64_t n, int32_t T, double dt, double F, const d
     m.dt = dt;
     m.F = F;
     m.p = 0;
-    cudaError_t e = l96_nl_launch(m, x0_dev, store_all ? traj_dev : nullptr, nullptr, nullptr, nullptr, nullptr,
-                                  store_all ? nullptr : traj_dev, (cudaStream_t)cuda_stream);
+    cudaError_t e = l96_nl_launch(m, x0_dev, store_all ? traj_dev : nullptr, nullptr, store_all ? nullptr : traj_dev,
+                                  (cudaStream_t)cuda_stream);
     return e == cudaSuccess ? RIOT_OK : RIOT_ECUDA;
 }
 
@@ -2604,7 +2681,7 @@ riot_status riot_psas(riot_ctx *ctx, int32_t m, int32_t q, int64_t sketch_stream
     CU(cudaMemcpyAsync(ctx->tmp, ctx->v, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     CU(scal(n, -1.0, ctx->tmp, s));
     if (ctx->model == RIOT_MODEL_ADVDIFF) CU(adv_tl_obs(ctx->a, ctx->tmp, ctx->psR, s));
-    else CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, ctx->tmp, nullptr, n, 1, 0, ctx->psR, 2, s));
+    else CU(l96_f64(ctx, ctx->tmp, nullptr, n, 1, 0, ctx->psR, 2));
     CU(mul(p, ctx->psS, ctx->d, ctx->psr, s));                 // S (H(x) - y)
     CU(mul(p, ctx->psSig, ctx->psR, ctx->psw, s));             // S b' = sigma_o (R^-1 b')
     CU(axpby(p, -1.0, ctx->psw, -1.0, ctx->psr, s));           // r = -S (H(x) - y) - S b'
@@ -2665,7 +2742,7 @@ riot_status riot_psas(riot_ctx *ctx, int32_t m, int32_t q, int64_t sketch_stream
     CU(mul(p, ctx->psS, ctx->psw, ctx->psF, s));               // dw = S w
     // x = x_b + B H^T dw = x_b + L v with v = L^T H^T dw (one adjoint run); dv = v_new - v
     if (ctx->model == RIOT_MODEL_ADVDIFF) CU(adv_ad_obs(ctx->a, ctx->psF, ctx->tmp, s));
-    else CU(l96_hvp_launch_f64(ctx->m, ctx->coef64, nullptr, ctx->tmp, n, 1, 0, ctx->psF, 1, s));
+    else CU(l96_f64(ctx, nullptr, ctx->tmp, n, 1, 0, ctx->psF, 1));
     CU(cudaMemcpyAsync(ctx->dv, ctx->tmp, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     CU(axpby(n, -1.0, ctx->v, 1.0, ctx->dv, s));
     CU(cudaMemcpyAsync(ctx->v, ctx->tmp, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));

@@ -50,6 +50,18 @@ struct Band {
 // ---------------------------------------------------------------------------
 // Lorenz-96 kernels (l96.cu)
 // ---------------------------------------------------------------------------
+// Tables and workspace of the FP64 integrations with the state split over CTAs (l96_split.cu).
+struct SplitWork {
+    int cols = 0;                    // columns the workspace holds (0: none)
+    int nrow = 0, last_step = -1;    // observed steps; the last of them
+    std::vector<int> orow_h;         // [T+1] row of step t among the observed steps, -1 if none (host)
+    const int *rowstep = nullptr;    // [nrow] its inverse
+    const int *obsrow = nullptr;     // [p] row of each observation
+    const double *wgt = nullptr;     // [nrow][n] sum of 1/sigma^2 over the observations of a variable
+    double *rows = nullptr;          // [cols][nrow][n]
+    double *a = nullptr, *b = nullptr;   // [cols][n] states
+};
+
 struct L96Dev {
     ChunkGeom geom;
     int T = 0;
@@ -75,15 +87,29 @@ struct L96Dev {
     const int *ostart = nullptr;     // [observed steps][Tp+1] first sorted observation of each chunk
     const int *osslot = nullptr;     // [p] slot of each sorted observation
     const int *osperm = nullptr;     // [p] index of each sorted observation in the caller's order
+    SplitWork sp;
 };
 
-// Nonlinear FP64 trajectory of one state; writes traj (T+1)*n (natural
-// layout, may be null), stage coefficients (may be null): double2 by slot
-// t*E + j, and float2 interleaved by element pair ((j/2)*Tp + t as float4),
-// the innovation d = H(x) - y (may be null) and 1/2 sum d^2/sigma^2 into
-// *jo (may be null, accumulated with atomicAdd: zero it first).
-cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, float2 *coef32,
-                          double2 *coef64, double *d, double *jo, double *xT, cudaStream_t s);
+// Nonlinear FP64 trajectory of one state (l96_split.cu): traj (T+1)*n, or only the final
+// state into xT (which x0 must not alias) when traj is null, and the stage coefficients
+// (double2 by slot t*E + j; may be null; the padding slots of short chunks are not written).
+cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, double2 *coef64, double *xT, cudaStream_t s);
+// FP32 copy of the stage coefficients, interleaved by element pair ((j/2)*Tp + t as float4)
+cudaError_t l96_coef32(const L96Dev &m, const double2 *coef64, float2 *coef32, cudaStream_t s);
+// The innovation d = H(x) - y from the trajectory and 1/2 sum d^2/sigma^2 added to *jo; with
+// rows, R^-1 d becomes the forcing of l96_split_gradient (needs the split workspace).
+cudaError_t l96_innov(const L96Dev &m, const double *traj, double *d, double *jo, bool rows, cudaStream_t s);
+// b = L^T H^T R^-1 d after l96_innov(rows), and y = A z when z is given (sp.cols >= 2 then)
+cudaError_t l96_split_gradient(const L96Dev &m, const double2 *coef, double *b, const double *z, double *y,
+                               cudaStream_t s);
+// The modes of l96_hvp_launch_f64 on at most sp.cols columns (modes 1 and 2: one), each
+// column's state split over many CTAs; r is used in modes 1 and 2 only.
+cudaError_t l96_split_f64(const L96Dev &m, const double2 *coef, const double *W, double *Y, int64_t ld, int ncols,
+                          int add_identity, double *r, int mode, cudaStream_t s);
+// whether that is modelled to take less than other_us per RK4 step
+bool l96_split_better(const L96Dev &m, int ncols, double other_us);
+// columns per CTA of l96_hvp_launch_f64 (its result) and its modelled us per RK4 step
+double hvp_f64_plan(const ChunkGeom &g, int ncols, int *P_out);
 
 // Batched FP64 Hessian-vector product (register-loaded coefficients, layout
 // [T][4][Np] double2 by slot).  mode 0: Y = A W (+W); mode 1: adjoint only
@@ -142,9 +168,9 @@ cudaError_t hvp_batch_plan(const HvpBatchWindow *w, int nwin, int P_cap, int S, 
 cudaError_t hvp_batch_launch(const HvpBatchPlan &plan, cudaStream_t s);
 void hvp_batch_free(HvpBatchPlan *plan);
 
-// out = L in or L^T in (FP64), ncols columns (ld = n)
-cudaError_t bsqrt_launch(const L96Dev &m, const double *in, double *out, int transpose, int ncols,
-                         cudaStream_t s);
+// out = L in or L^T in (+ add, laid out as out; FP64), ncols columns
+cudaError_t bsqrt_launch(const L96Dev &m, const double *in, int64_t ldi, double *out, int64_t ldo, int transpose,
+                         int ncols, const double *add, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Tracer transport model (advdiff.cu)

@@ -91,47 +91,58 @@ __device__ __forceinline__ void tl_tend(const real (&s)[E], real (&k)[E], const 
         if (j == E - 1) xp1 = p1;
         else if (j == E - 2) xp1 = full ? s[E - 1] : p1;
         else xp1 = s[j + 1 < E ? j + 1 : 0];
-        k[j] = c.x * (xp1 - xm2) + c.y * xm1 - s[j];
+        k[j] = fma(c.x, xp1 - xm2, fma(c.y, xm1, -s[j]));
     }
     if (!full) k[E - 1] = real(0);
 }
 
-// AD tendency out = J(X)^T m.
+// AD tendency out = J(X)^T m: a_{j-1} m_{j-1} - a_{j+2} m_{j+2} + b_{j+1} m_{j+1} - m_j in three
+// operations (the products a m, b m and their sums would be five); cl points at the left
+// chunk's last coefficient pair, cr at the right chunk's first.
 template <typename real, int E>
 __device__ __forceinline__ void ad_tend(const real (&m)[E], real (&out)[E], const typename V2<real>::type *cf,
+                                        const typename V2<real>::type *cl, const typename V2<real>::type *cr,
                                         bool full, real *H, int nthr, int tid, int left, int right, int &hb)
 {
-    real pp[E], qq[E];
+    real *Hb = H + hb * 4 * nthr;
+    Hb[tid] = full ? m[E - 1] : m[E - 2];
+    Hb[nthr + tid] = m[0];
+    Hb[2 * nthr + tid] = m[1];
+    real ca[E], cb[E];
 #pragma unroll
     for (int j = 0; j < E; ++j) {
         typename V2<real>::type c = cf[j];
-        pp[j] = c.x * m[j];
-        qq[j] = c.y * m[j];
+        ca[j] = c.x;
+        cb[j] = c.y;
     }
-    real *Hb = H + hb * 4 * nthr;
-    Hb[tid] = full ? pp[E - 1] : pp[E - 2];
-    Hb[nthr + tid] = pp[0];
-    Hb[2 * nthr + tid] = pp[1];
-    Hb[3 * nthr + tid] = qq[0];
+    const real aL = cl->x, aR1 = cr[1].x;
+    const typename V2<real>::type cR0 = cr[0];
     __syncthreads();
-    real pm1 = Hb[left];
-    real pR0 = Hb[nthr + right];
-    real pR1 = Hb[2 * nthr + right];
-    real qR0 = Hb[3 * nthr + right];
+    const real mL = Hb[left], mR0 = Hb[nthr + right], mR1 = Hb[2 * nthr + right];
     hb ^= 1;
 #pragma unroll
     for (int j = 0; j < E; ++j) {
-        real pjm1 = (j == 0) ? pm1 : pp[j >= 1 ? j - 1 : 0];
-        real qjp1;
-        if (j <= E - 3) qjp1 = qq[j + 1 < E ? j + 1 : 0];
-        else if (j == E - 2) qjp1 = full ? qq[E - 1] : qR0;
-        else qjp1 = qR0;
-        real pjp2;
-        if (j <= E - 4) pjp2 = pp[j + 2 < E ? j + 2 : 0];
-        else if (j == E - 3) pjp2 = full ? pp[E - 1] : pR0;
-        else if (j == E - 2) pjp2 = full ? pR0 : pR1;
-        else pjp2 = pR1;
-        out[j] = pjm1 - pjp2 + qjp1 - m[j];
+        const real mm1 = (j == 0) ? mL : m[j >= 1 ? j - 1 : 0];
+        const real am1 = (j == 0) ? aL : ca[j >= 1 ? j - 1 : 0];
+        real mp1, bp1, mp2, ap2;
+        if (j <= E - 2 && (full || j <= E - 3)) {
+            mp1 = m[j + 1 < E ? j + 1 : 0];
+            bp1 = cb[j + 1 < E ? j + 1 : 0];
+        } else {
+            mp1 = mR0;
+            bp1 = cR0.y;
+        }
+        if (j <= E - 3 && (full || j <= E - 4)) {
+            mp2 = m[j + 2 < E ? j + 2 : 0];
+            ap2 = ca[j + 2 < E ? j + 2 : 0];
+        } else if (full ? (j == E - 2) : (j == E - 3)) {
+            mp2 = mR0;
+            ap2 = cR0.x;
+        } else {
+            mp2 = mR1;
+            ap2 = aR1;
+        }
+        out[j] = fma(am1, mm1, fma(-ap2, mp2, fma(bp1, mp1, -m[j])));
     }
     if (!full) out[E - 1] = real(0);
 }
@@ -187,9 +198,10 @@ __global__ void __launch_bounds__(512) l96_hvp_kernel(const HvpArgs<real> a)
     const int s0 = G.start(t);
     const int len = G.len(t);
     const bool full = (len == E);
+    const int tl = (t == 0) ? Tp - 1 : t - 1, tr = (t == Tp - 1) ? 0 : t + 1, lenL = G.len(tl);
     real *st = state + pp * SP;
     int hb = 0;
-    const real h = a.dt, h2 = real(0.5) * a.dt, h6 = a.dt / real(6), h3 = a.dt / real(3);
+    const real h = a.dt, h2 = real(0.5) * a.dt, h6 = a.dt / real(6);
     const size_t rbase = (size_t)(active ? probe : 0) * (size_t)a.p;
 
     real dx[E];
@@ -221,16 +233,16 @@ __global__ void __launch_bounds__(512) l96_hvp_kernel(const HvpArgs<real> a)
             for (int j = 0; j < E; ++j) s[j] = dx[j];
             tl_tend<real, E>(s, k, cf, full, H, nthr, tid, left, right, hb);
 #pragma unroll
-            for (int j = 0; j < E; ++j) { acc[j] = k[j]; s[j] = dx[j] + h2 * k[j]; }
+            for (int j = 0; j < E; ++j) { acc[j] = k[j]; s[j] = fma(h2, k[j], dx[j]); }
             tl_tend<real, E>(s, k, cf + Np, full, H, nthr, tid, left, right, hb);
 #pragma unroll
-            for (int j = 0; j < E; ++j) { acc[j] += real(2) * k[j]; s[j] = dx[j] + h2 * k[j]; }
+            for (int j = 0; j < E; ++j) { acc[j] = fma(real(2), k[j], acc[j]); s[j] = fma(h2, k[j], dx[j]); }
             tl_tend<real, E>(s, k, cf + 2 * Np, full, H, nthr, tid, left, right, hb);
 #pragma unroll
-            for (int j = 0; j < E; ++j) { acc[j] += real(2) * k[j]; s[j] = dx[j] + h * k[j]; }
+            for (int j = 0; j < E; ++j) { acc[j] = fma(real(2), k[j], acc[j]); s[j] = fma(h, k[j], dx[j]); }
             tl_tend<real, E>(s, k, cf + 3 * Np, full, H, nthr, tid, left, right, hb);
 #pragma unroll
-            for (int j = 0; j < E; ++j) { acc[j] += k[j]; dx[j] = dx[j] + h6 * acc[j]; }
+            for (int j = 0; j < E; ++j) { acc[j] += k[j]; dx[j] = fma(h6, acc[j], dx[j]); }
         }
         if (a.mode == 2) return;
     }
@@ -252,22 +264,23 @@ __global__ void __launch_bounds__(512) l96_hvp_kernel(const HvpArgs<real> a)
             for (int j = 0; j < E; ++j) lam[j] = (j < len) ? st[sw(t * E + j)] : real(0);
         }
         if (tt == 0) break;
-        const typename V2<real>::type *cf = a.coef + (size_t)(tt - 1) * 4 * Np + t * E;
-        real lk[E], ls[E], lx[E];
+        // lam_0 = lam + l4 + l3 + l2 + l1 with mu = (h / 6) lam, l4 = J4^T mu, l3 = 2 n3, n3 =
+        // J3^T (mu + (h / 2) l4), l2 = 2 n2, n2 = J2^T (mu + (h / 2) n3), l1 = J1^T (mu + h n2)
+        const typename V2<real>::type *cs = a.coef + (size_t)(tt - 1) * 4 * Np;
+        const int oL = tl * E + lenL - 1, oR = tr * E;
+        real mu[E], m[E], k[E];
 #pragma unroll
-        for (int j = 0; j < E; ++j) lk[j] = h6 * lam[j];
-        ad_tend<real, E>(lk, ls, cf + 3 * Np, full, H, nthr, tid, left, right, hb);
+        for (int j = 0; j < E; ++j) m[j] = mu[j] = h6 * lam[j];
 #pragma unroll
-        for (int j = 0; j < E; ++j) { lx[j] = lam[j] + ls[j]; lk[j] = h3 * lam[j] + h * ls[j]; }
-        ad_tend<real, E>(lk, ls, cf + 2 * Np, full, H, nthr, tid, left, right, hb);
+        for (int st = 3; st >= 0; --st) {
+            const typename V2<real>::type *c = cs + st * Np;
+            ad_tend<real, E>(m, k, c + t * E, c + oL, c + oR, full, H, nthr, tid, left, right, hb);
 #pragma unroll
-        for (int j = 0; j < E; ++j) { lx[j] += ls[j]; lk[j] = h3 * lam[j] + h2 * ls[j]; }
-        ad_tend<real, E>(lk, ls, cf + Np, full, H, nthr, tid, left, right, hb);
-#pragma unroll
-        for (int j = 0; j < E; ++j) { lx[j] += ls[j]; lk[j] = h6 * lam[j] + h2 * ls[j]; }
-        ad_tend<real, E>(lk, ls, cf, full, H, nthr, tid, left, right, hb);
-#pragma unroll
-        for (int j = 0; j < E; ++j) lam[j] = lx[j] + ls[j];
+            for (int j = 0; j < E; ++j) {
+                lam[j] = (st == 0 || st == 3) ? lam[j] + k[j] : fma(real(2), k[j], lam[j]);
+                if (st > 0) m[j] = fma(st == 1 ? h : h2, k[j], mu[j]);
+            }
+        }
     }
 
     // ---- epilogue: y = L^T lambda_0 = S diag(sigma) lambda_0 (+ w) ----
@@ -285,6 +298,29 @@ __global__ void __launch_bounds__(512) l96_hvp_kernel(const HvpArgs<real> a)
         for (int j = 0; j < E; ++j)
             if (j < len) yo[s0 + j] = y[j] + ((a.add_identity && w) ? w[s0 + j] : real(0));
     }
+}
+
+// Columns per CTA of the FP64 kernel and its modelled time per RK4 step.  The kernel is bound by
+// FP64 issue, one warp instruction per 64 cycles and SM sub-partition, so what counts is the
+// largest number of warps that a sub-partition gets: few columns per CTA spread over all SMs
+// (128 columns of 1000 variables: 32 CTAs of four columns 3.5 ms, 128 CTAs of one 0.7 ms), more
+// where a column alone leaves most of a warp's lanes idle.
+double hvp_f64_plan(const ChunkGeom &g, int ncols, int *P_out)
+{
+    int Pmax = 512 / g.Tp;
+    if (Pmax > ncols) Pmax = ncols;
+    if (Pmax > 64) Pmax = 64;
+    const int sms = num_sms();
+    long long best = -1;
+    for (int P = 1; P <= Pmax; ++P) {
+        const long long ctas = (ncols + P - 1) / P, warps = (P * g.Tp + 31) / 32;
+        const long long load = ((ctas + sms - 1) / sms * warps + 3) / 4;
+        if (best < 0 || load < best) {
+            best = load;
+            *P_out = P;
+        }
+    }
+    return 0.85 * (double)best * g.E;
 }
 
 template <typename real>
@@ -314,10 +350,9 @@ static cudaError_t hvp_launch(const L96Dev &m, const typename V2<real>::type *co
     a.r = r;
     a.ld = ld;
     const int Tp = m.geom.Tp;
-    int P = 512 / Tp;
+    int P = 0;
+    hvp_f64_plan(m.geom, ncols, &P);
     if (P < 1) return cudaErrorInvalidConfiguration;
-    if (P > ncols) P = ncols;
-    if (P > 64) P = 64;
     a.P = P;
     const int nthr = P * Tp;
     const size_t sm = sizeof(real) * (8 * (size_t)nthr + (size_t)P * stage_pad(m.geom.Np));
@@ -350,193 +385,51 @@ cudaError_t l96_hvp_launch_f64(const L96Dev &m, const double2 *coef, const doubl
 }
 
 // ---------------------------------------------------------------------------
-// Nonlinear FP64 trajectory + stage coefficients + innovation (one CTA).
+// Standalone L / L^T application in FP64 (outer-loop update, covariance, split integrations).
+// A block of 64 threads forms 64 outputs of one column from a window of the column in shared
+// memory (scaled there for L^T: one product per value instead of one per tap).
 // ---------------------------------------------------------------------------
-struct NlArgs {
-    ChunkGeom geom;
-    int T, p;
-    double dt, F;
-    const int *optr, *oslot;
-    const double *y, *rinv, *x0;
-    double *traj, *d, *jo, *xT;
-    float2 *coef32;
-    double2 *coef64;
-};
+constexpr int kBsqrtBlock = 64;
 
-template <int E>
-__global__ void __launch_bounds__(512) l96_nl_kernel(const NlArgs a)
+__global__ void __launch_bounds__(kBsqrtBlock) bsqrt_kernel(int n, int hl, int hh, const double *band, const double *sig,
+                                                            const double *in, long long ldi, double *out,
+                                                            long long ldo, int transpose, const double *add)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double *H = reinterpret_cast<double *>(smem_raw);
-    const int nthr = blockDim.x;
-    double *st = H + 8 * nthr;
-    const ChunkGeom &G = a.geom;
-    const int Np = G.Np, n = G.n, Tp = G.Tp;
-    const int t = threadIdx.x, tid = threadIdx.x;
-    const int left = (t == 0) ? Tp - 1 : t - 1, right = (t == Tp - 1) ? 0 : t + 1;
-    const int s0 = G.start(t), len = G.len(t);
-    const bool full = (len == E);
-    int hb = 0;
-    const double h = a.dt, h2 = 0.5 * a.dt, h6 = a.dt / 6.0, F = a.F;
-    double jsum = 0.0;
-
-    double x[E];
-#pragma unroll
-    for (int j = 0; j < E; ++j) x[j] = (j < len) ? a.x0[s0 + (j < len ? j : 0)] : 0.0;
-
-    for (int tt = 0;; ++tt) {
-        if (a.traj) {
-#pragma unroll
-            for (int j = 0; j < E; ++j)
-                if (j < len) a.traj[(size_t)tt * n + s0 + j] = x[j];
-        }
-        const int o0 = a.p ? a.optr[tt] : 0, o1 = a.p ? a.optr[tt + 1] : 0;
-        if (o0 < o1) {
-#pragma unroll
-            for (int j = 0; j < E; ++j) st[sw(t * E + j)] = x[j];
-            __syncthreads();
-            for (int o = o0 + t; o < o1; o += Tp) {
-                double dd = st[sw(a.oslot[o])] - a.y[o];
-                if (a.d) a.d[o] = dd;
-                jsum += 0.5 * dd * dd * a.rinv[o];
-            }
-            __syncthreads();
-        }
-        if (tt == a.T) break;
-        double X[E], acc[E];
-#pragma unroll
-        for (int j = 0; j < E; ++j) X[j] = x[j];
-#pragma unroll 1
-        for (int stage = 0; stage < 4; ++stage) {
-            double m2, m1, p1;
-            xchg_tl<double, E>(X, full, H, nthr, tid, left, right, hb, m2, m1, p1);
-            double f[E];
-            const size_t cbase = ((size_t)tt * 4 + stage) * Np + (size_t)t * E;
-#pragma unroll
-            for (int j = 0; j < E; ++j) {
-                double xm2 = (j == 0) ? m2 : (j == 1 ? m1 : X[j >= 2 ? j - 2 : 0]);
-                double xm1 = (j == 0) ? m1 : X[j >= 1 ? j - 1 : 0];
-                double xp1;
-                if (j == E - 1) xp1 = p1;
-                else if (j == E - 2) xp1 = full ? X[E - 1] : p1;
-                else xp1 = X[j + 1 < E ? j + 1 : 0];
-                double ca = xm1, cb = xp1 - xm2;
-                f[j] = cb * ca - X[j] + F;
-                if (j == E - 1 && !full) { ca = 0.0; cb = 0.0; f[j] = 0.0; }
-                // FP32 copy interleaved by element pair across threads: float4 index
-                // (j / 2) * Tp + t within the stage, so that the FP32 kernel's
-                // shared-memory reads of one pair are contiguous across threads
-                if (a.coef32)
-                    a.coef32[((size_t)tt * 4 + stage) * Np + (size_t)(j >> 1) * 2 * Tp + 2 * t + (j & 1)] =
-                        make_float2((float)ca, (float)cb);
-                if (a.coef64) a.coef64[cbase + j] = make_double2(ca, cb);
-            }
-            const double c = (stage == 2) ? h : h2;
-            const double wgt = (stage == 0 || stage == 3) ? 1.0 : 2.0;
-#pragma unroll
-            for (int j = 0; j < E; ++j) {
-                acc[j] = (stage == 0) ? f[j] : acc[j] + wgt * f[j];
-                X[j] = x[j] + c * f[j];
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < E; ++j) x[j] = full || j < E - 1 ? x[j] + h6 * acc[j] : 0.0;
+    extern __shared__ double sm_band[];
+    const int i0 = blockIdx.x * kBsqrtBlock, i = i0 + threadIdx.x;
+    const double *x = in + (size_t)blockIdx.y * ldi;
+    const int width = kBsqrtBlock + hl + hh;
+    for (int w = threadIdx.x; w < width; w += kBsqrtBlock) {
+        int ii = (i0 + w - hl) % n;
+        ii += (ii < 0) ? n : 0;
+        sm_band[w] = transpose ? sig[ii] * x[ii] : x[ii];
     }
-    if (a.xT) {
-#pragma unroll
-        for (int j = 0; j < E; ++j)
-            if (j < len) a.xT[s0 + j] = x[j];
-    }
-    if (a.jo) {
-        // block reduction of jsum
-        __syncthreads();
-        for (int off = 16; off > 0; off >>= 1) jsum += __shfl_down_sync(0xffffffffu, jsum, off);
-        if ((tid & 31) == 0) st[tid >> 5] = jsum;
-        __syncthreads();
-        if (tid == 0) {
-            double s = 0.0;
-            for (int w = 0; w < (nthr + 31) / 32; ++w) s += st[w];
-            atomicAdd(a.jo, s);
-        }
-    }
+    __syncthreads();
+    if (i >= n) return;
+    double acc = 0.0;
+    for (int d = 0; d <= hl + hh; ++d) acc = fma(band[d], sm_band[threadIdx.x + d], acc);
+    double y = transpose ? acc : sig[i] * acc;
+    if (add) y += add[(size_t)blockIdx.y * ldo + i];
+    out[(size_t)blockIdx.y * ldo + i] = y;
 }
 
-cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, float2 *coef32, double2 *coef64,
-                          double *d, double *jo, double *xT, cudaStream_t s)
-{
-    NlArgs a;
-    a.geom = m.geom;
-    a.T = m.T;
-    a.p = m.p;
-    a.dt = m.dt;
-    a.F = m.F;
-    a.optr = m.optr;
-    a.oslot = m.oslot;
-    a.y = m.y;
-    a.rinv = m.rinv64;
-    a.x0 = x0;
-    a.traj = traj;
-    a.d = d;
-    a.jo = jo;
-    a.xT = xT;
-    a.coef32 = coef32;
-    a.coef64 = coef64;
-    const int nthr = m.geom.Tp;
-    if (nthr > 512) return cudaErrorInvalidConfiguration;
-    const size_t sm = sizeof(double) * (8 * (size_t)nthr + stage_pad(m.geom.Np));
-    cudaError_t e = cudaSuccess;
-    switch (m.geom.E) {
-    case 4:
-        e = cudaFuncSetAttribute(l96_nl_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_nl_kernel<4><<<1, nthr, sm, s>>>(a); }
-        break;
-    case 8:
-        e = cudaFuncSetAttribute(l96_nl_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_nl_kernel<8><<<1, nthr, sm, s>>>(a); }
-        break;
-    case 16:
-        e = cudaFuncSetAttribute(l96_nl_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_nl_kernel<16><<<1, nthr, sm, s>>>(a); }
-        break;
-    default:
-        return cudaErrorInvalidValue;
-    }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------
-// Standalone L / L^T application in FP64 (outer-loop update, covariance).
-// ---------------------------------------------------------------------------
-__global__ void bsqrt_kernel(int n, int ncols, int hl, int hh, const double *band, const double *sig,
-                             const double *in, double *out, int transpose)
-{
-    const int64_t total = (int64_t)n * ncols;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int col = (int)(idx / n), i = (int)(idx - (int64_t)col * n);
-        const double *x = in + (size_t)col * n;
-        double acc = 0.0;
-        for (int d = -hl; d <= hh; ++d) {
-            int ii = i + d;
-            ii += (ii < 0) ? n : 0;
-            ii -= (ii >= n) ? n : 0;
-            acc += band[d + hl] * (transpose ? sig[ii] * x[ii] : x[ii]);
-        }
-        out[(size_t)col * n + i] = transpose ? acc : sig[i] * acc;
-    }
-}
-
-cudaError_t bsqrt_launch(const L96Dev &m, const double *in, double *out, int transpose, int ncols, cudaStream_t s)
+cudaError_t bsqrt_launch(const L96Dev &m, const double *in, int64_t ldi, double *out, int64_t ldo, int transpose,
+                         int ncols, const double *add, cudaStream_t s)
 {
     if (ncols <= 0) return cudaSuccess;
-    const int64_t total = (int64_t)m.geom.n * ncols;
-    int blocks = (int)((total + 255) / 256);
-    if (blocks > 4096) blocks = 4096;
-    count_launch();
-    bsqrt_kernel<<<blocks, 256, 0, s>>>(m.geom.n, ncols, m.band.hl, m.band.hh, m.band64, m.sig64, in, out,
-                                        transpose);
-    return cudaGetLastError();
+    const int n = m.geom.n;
+    const size_t sm = sizeof(double) * (kBsqrtBlock + m.band.hl + m.band.hh);   // at most 64 + 8191 values
+    cudaError_t e = cudaFuncSetAttribute(bsqrt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    for (int c0 = 0; c0 < ncols; c0 += 65535) {
+        const dim3 grid((n + kBsqrtBlock - 1) / kBsqrtBlock, ncols - c0 < 65535 ? ncols - c0 : 65535);
+        count_launch();
+        bsqrt_kernel<<<grid, kBsqrtBlock, sm, s>>>(n, m.band.hl, m.band.hh, m.band64, m.sig64, in + (size_t)c0 * ldi, ldi,
+                                                   out + (size_t)c0 * ldo, ldo, transpose,
+                                                   add ? add + (size_t)c0 * ldo : nullptr);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace riot
