@@ -21,6 +21,8 @@
 // u1..u3, accumulated at level 0 for the emission blocks.
 #include <cuda_runtime.h>
 #include <math.h>
+#include <stdint.h>
+#include <string.h>
 
 #include "internal.h"
 
@@ -149,14 +151,297 @@ __global__ void __launch_bounds__((TX + 2 * kHalo) * (TY + 2 * kHalo), 1) adv_st
     }
 }
 
-// FP32 stepper: nested RK4 on pairs of levels with packed FP32x2 arithmetic.  For the
+// FP32 stepper: nested RK4 marching through the levels, packed FP32x2 arithmetic.  For the
 // linear autonomous tendency f(w) = A w + s of one step, RK4 gives c+ = P(hA) c + h Q(hA) s,
 // P and Q the Taylor polynomials of degree 4 and 3 of exp(z) and (exp(z) - 1) / z.  Nested
-// (Horner), that is w <- c + a (A w + s) for a = h/4, h/3, h/2, h from w = c, the last w being
+// (Horner), that is w_{s+1} = c + a_s (A w_s + s) for a = h/4, h/3, h/2, h from w_0 = c, w_4 being
 // c+: the same four applications of A as the classical stages, with one state array besides
 // c instead of two.  The adjoint P(hA^T) lam is the same recursion with A^T and no source;
 // the input of its last stage is Q(hA^T) lam, so the source adjoint is h times its level 0.
-// Levels are held in pairs (2p, 2p + 1) (padded with zero coefficients beyond nz) and
+//
+// A CTA of NW warps owns a region of 64 columns in x by RW NW rows in y of one probe, of which
+// the inner 56 x (RW NW - 8) are its tile; a warp holds RW rows, a lane two neighbouring columns
+// of each as one register pair (every operation serves both).  Iteration k computes level k - 1 - s of
+// stage s for all four stages: a stage needs its input one level up (computed earlier in the
+// same iteration), one level down and at the four horizontal neighbours, so three levels per
+// stage stay in registers and only one level per stage is published in shared memory (a warp's
+// outer rows), by one barrier per iteration.  East and west neighbours come from the lane's own
+// pair and two shuffles, a row's north and south neighbours from the warp's other rows.  The
+// field's levels arrive by asynchronous copies three levels ahead; its level -1 holds the
+// source, which enters level 0 as the neighbour below with coefficient 1.
+//
+// Bound: register ports and shared memory together.  A packed FMA of three different register
+// pairs takes 3 cycles of its sub-partition (2 with one of them reused, hence the order of the
+// operations over a warp's rows); the 10 packed operations of a pair and stage make 80 us of the
+// 192 x 192 x 30, 32-column step with the halo's recomputation (64 x 36 regions, 76 % of the rows
+// and 75 % of the columns owned), the shared-memory pipe 55 % of the time.  Measured: 262 -> 182
+// us per step (column form -> this), 32 columns of 240 steps 132.8 -> 90.4 ms, with the same
+// error.  Slower: 16 warps of two rows (97 ms), 8 of four (98 ms), scalar east and west products
+// (mixed with packed ones they stall, 103 ms), barrier before the copies (97 ms).  Coefficients
+// multiplied by a_s beforehand save nothing and round the balance of the vertical fluxes (error
+// 2 to 5e-7).
+constexpr int kZW = 64;             // columns of a region
+constexpr int kZTX = kZW - 2 * kHalo;
+constexpr int kZLevels = kMaxNZ + 6;
+
+struct StepArgsZ {
+    unsigned long long al[4];                                 // h/4, h/3, h/2, h, each twice
+    float amp[kMaxNZ], ku[kMaxNZ], kl[kMaxNZ], nkd[kMaxNZ];   // 0 beyond nz
+    const float *cin;
+    float *cout;
+    long long pstride;
+    const float *src;
+    long long sstride;
+    float *ebar;
+    long long estride;
+    const float *u, *v;
+    int nx, ny, nz;
+    float h, rdx, rdy;
+};
+
+// Upwind coefficients of one column: self, east, west, north, south (0 outside the walls).
+template <bool ADJ>
+__device__ __forceinline__ void column_coefs(const StepArgsZ &a, int gx, int gy, float (&cf)[5])
+{
+#pragma unroll
+    for (int i = 0; i < 5; ++i) cf[i] = 0.f;
+    if (gy < 0 || gy >= a.ny) return;
+    const size_t row = (size_t)gy * a.nx, col = row + gx;
+    const float uL = a.u[col], uR = a.u[row + (gx + 1 == a.nx ? 0 : gx + 1)];
+    const float vS = a.v[col], vN = a.v[col + a.nx];
+    const float uLp = fmaxf(uL, 0.f), uLm = fminf(uL, 0.f);
+    const float uRp = fmaxf(uR, 0.f), uRm = fminf(uR, 0.f);
+    const float vSp = fmaxf(vS, 0.f), vSm = fminf(vS, 0.f);
+    const float vNp = fmaxf(vN, 0.f), vNm = fminf(vN, 0.f);
+    cf[0] = (uLm - uRp) * a.rdx + (vSm - vNp) * a.rdy;
+    cf[1] = ADJ ? uRp * a.rdx : -uRm * a.rdx;
+    cf[2] = ADJ ? -uLm * a.rdx : uLp * a.rdx;
+    cf[3] = ADJ ? vNp * a.rdy : -vNm * a.rdy;
+    cf[4] = ADJ ? -vSm * a.rdy : vSp * a.rdy;
+}
+
+// A pair of neighbouring columns in one 64-bit register.
+using pair_t = unsigned long long;
+
+__device__ __forceinline__ pair_t pk(float x, float y)
+{
+    pair_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 upk(pair_t p)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c)
+{
+    pair_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ pair_t mul2(pair_t a, pair_t b)
+{
+    pair_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// asynchronous copy of BYTES (4 or 8) to shared memory, zeros when !in
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void *dst, const float *src, bool in)
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = in ? BYTES : 0;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(BYTES), "r"(n) : "memory");
+}
+
+constexpr int kZRing = 6;   // levels of the field in shared memory (the unrolling, so that slots are constants)
+constexpr int kZAhead = 3;  // levels copied ahead of the iteration that reads them
+
+// PAIR: nx is even and the fields are 8-byte aligned, so that a lane's two columns are one access.
+template <int NW, int RW, bool ADJ, bool PAIR>
+__global__ void __launch_bounds__(32 * NW) adv_step_z_kernel(const __grid_constant__ StepArgsZ a)
+{
+    constexpr int ROWS = RW * NW, TY = ROWS - 2 * kHalo;
+    extern __shared__ __align__(16) unsigned char advz_smem[];
+    // the field's levels (also the published input of stage 0): [kZRing][ROWS][32]; published
+    // inputs of stages 1..3: [2][3][ROWS][32]; level coefficients, each twice (for both columns
+    // of a pair): (amp, ku), (kl, nkd) of level z at z + 3, zeros below and from level nz on
+    pair_t(*F)[ROWS][32] = reinterpret_cast<pair_t(*)[ROWS][32]>(advz_smem);
+    pair_t(*S)[3][ROWS][32] = reinterpret_cast<pair_t(*)[3][ROWS][32]>(F + kZRing);
+    ulonglong2(*LC)[2] = reinterpret_cast<ulonglong2(*)[2]>(S + 2);
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int x0 = blockIdx.x * kZTX, y0 = blockIdx.y * TY;
+    const int ix = 2 * lane - kHalo;
+    int gx0 = (x0 + ix) % nx;
+    if (gx0 < 0) gx0 += nx;
+    const int gx1 = gx0 + 1 == nx ? 0 : gx0 + 1;
+    const int plane = nx * ny;
+    const float *cin = a.cin + (size_t)blockIdx.z * a.pstride;
+    const int ry0 = RW * wp, sN = min(ry0 + RW, ROWS - 1), sS = max(ry0 - 1, 0);
+
+    bool valid[RW], mine[RW];
+    int row0[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+        const int gy = y0 - kHalo + ry0 + r;
+        valid[r] = gy >= 0 && gy < ny;
+        row0[r] = valid[r] ? gy * nx : 0;
+        mine[r] = valid[r] && ry0 + r >= kHalo && ry0 + r < kHalo + TY && ix >= 0 && ix < kZTX && x0 + ix < nx;
+    }
+    // copy of level z (slot z mod kZRing); beyond the last level zeros, from an address in range
+    auto fetch = [&](int z, int slot) {
+        const float *lev = cin + (size_t)min(z, nz - 1) * plane;
+        const bool top = z < nz;
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+            float *d = reinterpret_cast<float *>(&F[slot][ry0 + r][lane]);
+            copy_async<PAIR ? 8 : 4>(d, lev + (row0[r] + gx0), valid[r] && top);
+            if (!PAIR) copy_async<4>(d + 1, lev + (row0[r] + gx1), valid[r] && top);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int z = 0; z < kZAhead; ++z) fetch(z, z);
+    for (int i = threadIdx.x; i < kZLevels; i += 32 * NW) {
+        const int z = i - 3, zz = z >= 0 && z < nz ? z : 0;
+        const float f = z >= 0 && z < nz ? 1.f : 0.f;
+        const float am = f * a.amp[zz], u = f * a.ku[zz], l = z == 0 ? 1.f : f * a.kl[zz], d = f * a.nkd[zz];
+        LC[i][0] = make_ulonglong2(pk(am, am), pk(u, u));
+        LC[i][1] = make_ulonglong2(pk(l, l), pk(d, d));
+    }
+    pair_t C[RW][5];   // self, east, west, north, south
+    float2 e0[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+        const int gy = y0 - kHalo + ry0 + r;
+        float c0[5], c1[5];
+        column_coefs<ADJ>(a, gx0, gy, c0);
+        column_coefs<ADJ>(a, gx1, gy, c1);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) C[r][i] = pk(c0[i], c1[i]);
+        e0[r] = make_float2(0.f, 0.f);
+    }
+
+    // W[s][z mod 3][r]: input of stage s at level z; c3, c4: the field three and four levels back
+    pair_t W[4][3][RW], c3[RW], c4[RW];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int r = 0; r < RW; ++r) W[s][i][r] = 0;
+    // the source enters level 0 of every stage as a level -1 that holds it, with coefficient 1
+    // (kl of level 0, which has no neighbour below)
+    if (!ADJ && a.src)
+#pragma unroll
+        for (int r = 0; r < RW; ++r)
+            if (valid[r]) {
+                const float *sp = a.src + (size_t)blockIdx.z * a.sstride + row0[r];
+                W[0][2][r] = W[1][2][r] = pk(sp[gx0], sp[gx1]);
+            }
+    asm volatile("cp.async.wait_group %0;" ::"n"(kZAhead - 1) : "memory");
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+        c3[r] = c4[r] = 0;
+        W[0][0][r] = F[0][ry0 + r][lane];
+    }
+    float *cout = a.cout + (size_t)blockIdx.z * a.pstride;
+
+    for (int k0 = 1; k0 < nz + 4; k0 += 6) {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const int k = k0 + j;        // k = j + 1 (mod 6)
+            if (k >= nz + 4) break;
+            pair_t(*Sk)[ROWS][32] = S[(j + 1) & 1];
+            // publish level k - 1 - s of the inputs of stages 1..3
+#pragma unroll
+            for (int s = 1; s < 4; ++s)
+#pragma unroll
+                for (int r = 0; r < RW; r += RW - 1) Sk[s - 1][ry0 + r][lane] = W[s][(j + 6 - s) % 3][r];
+            fetch(k + kZAhead - 1, (j + kZAhead) % kZRing);
+            asm volatile("cp.async.wait_group %0;" ::"n"(kZAhead - 1) : "memory");   // level k is here
+#pragma unroll
+            for (int r = 0; r < RW; ++r) {
+                c4[r] = c3[r];
+                c3[r] = W[0][(j + 1) % 3][r];
+                W[0][(j + 1) % 3][r] = F[(j + 1) % kZRing][ry0 + r][lane];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const int z = k - 1 - s;
+                const int im = (j + 6 - s) % 3, iu = (im + 1) % 3, id = (im + 2) % 3;
+                const ulonglong2 l0 = LC[z + 3][0], l1 = LC[z + 3][1];
+                const pair_t al = a.al[s];
+                const pair_t(*P)[32] = s == 0 ? F[j] : Sk[s > 0 ? s - 1 : 0];   // level z of stage 0: k - 1 = j (mod 6)
+                const pair_t nN = P[sN][lane], nS = P[sS][lane];
+                float *lev = cout + (ptrdiff_t)z * plane;
+                // operations with the same coefficient next to each other: a packed operation with
+                // three different register pairs takes 3 cycles, with one of them kept 2
+                pair_t q[RW];
+#pragma unroll
+                for (int r = 0; r < RW; ++r) {
+                    const pair_t wo = W[s][im][r];
+                    const float2 w = upk(wo);
+                    const float wE = __shfl_down_sync(0xffffffffu, w.x, 1), wW = __shfl_up_sync(0xffffffffu, w.y, 1);
+                    const pair_t N = r + 1 < RW ? W[s][im][r + 1 < RW ? r + 1 : 0] : nN;
+                    const pair_t So = r > 0 ? W[s][im][r > 0 ? r - 1 : 0] : nS;
+                    q[r] = mul2(C[r][0], wo);
+                    q[r] = fma2(C[r][1], pk(w.y, wE), q[r]);
+                    q[r] = fma2(C[r][2], pk(wW, w.x), q[r]);
+                    q[r] = fma2(C[r][3], N, q[r]);
+                    q[r] = fma2(C[r][4], So, q[r]);
+                }
+#pragma unroll
+                for (int r = 0; r < RW; ++r) q[r] = mul2(l0.x, q[r]);
+#pragma unroll
+                for (int r = 0; r < RW; ++r) q[r] = fma2(l1.y, W[s][im][r], q[r]);
+#pragma unroll
+                for (int r = 0; r < RW; ++r) q[r] = fma2(l1.x, W[s][id][r], q[r]);
+#pragma unroll
+                for (int r = 0; r < RW; ++r) q[r] = fma2(l0.y, W[s][iu][r], q[r]);
+#pragma unroll
+                for (int r = 0; r < RW; ++r) {
+                    const pair_t wo = W[s][im][r];
+                    const pair_t wn = fma2(al, q[r], s < 2 ? W[0][im][r] : s == 2 ? c3[r] : c4[r]);
+                    if (s < 3) {
+                        W[s + 1][im][r] = wn;   // level z (mod 3 as im)
+                    } else {
+                        if (ADJ && j == 3 && k0 == 1) {   // z = 0
+                            const float2 e = upk(wo);
+                            e0[r] = e;
+                        }
+                        if (mine[r] && (j >= 3 || k0 > 1)) {   // 0 <= z < nz, as 4 <= k < nz + 4
+                            float *o = lev + row0[r];
+                            if (PAIR) {
+                                *reinterpret_cast<pair_t *>(o + gx0) = wn;
+                            } else {
+                                const float2 t = upk(wn);
+                                o[gx0] = t.x;
+                                if (x0 + ix + 1 < nx) o[gx1] = t.y;
+                            }
+                        }
+                    }
+                }
+            }
+        }
+    }
+    if (ADJ && a.ebar)
+#pragma unroll
+        for (int r = 0; r < RW; ++r)
+            if (mine[r]) {
+                float *e = a.ebar + (size_t)blockIdx.z * a.estride + row0[r];
+                e[gx0] += a.h * e0[r].x;
+                if (PAIR || x0 + ix + 1 < nx) e[gx1] += a.h * e0[r].y;
+            }
+}
+
+// FP32 stepper for few columns of the sketch: the recursion of adv_step_z_kernel with whole
+// columns of levels in registers, four barriers per step on 32 x 8 tiles: four times the CTAs
+// of the level-marching form, each done in a quarter of its time.  Levels are held in pairs (2p, 2p + 1) (padded with zero coefficients beyond nz) and
 // combined by packed FP32x2 instructions, one instruction for two levels; the shared planes
 // hold the pairs, so a horizontal neighbour fetch is one 64-bit load for two levels.  (Pairs
 // (p, p + NZP), whose vertical neighbours are whole pairs, measured slower: the renamed
@@ -481,6 +766,24 @@ cudaError_t step_nz(const StepArgs<R> &a, int P, cudaStream_t s)
     return cudaGetLastError();
 }
 
+template <int NW, int RW, bool ADJ, bool PAIR>
+cudaError_t step_z_launch(const StepArgsZ &a, int P, cudaStream_t s)
+{
+    constexpr int TY = RW * NW - 2 * kHalo;
+    const size_t smem = sizeof(pair_t) * (kZRing + 2 * 3) * RW * NW * 32 + sizeof(ulonglong2) * 2 * kZLevels;
+    auto kern = adv_step_z_kernel<NW, RW, ADJ, PAIR>;
+    static bool attr_done = false;
+    if (!attr_done) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr_done = true;
+    }
+    dim3 grid((a.nx + kZTX - 1) / kZTX, (a.ny + TY - 1) / TY, P);
+    kern<<<grid, 32 * NW, smem, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
 template <int NZP, int TX, int TY, bool ADJ>
 cudaError_t step_f2_nz(const StepArgsF2 &a, int P, cudaStream_t s)
 {
@@ -499,12 +802,9 @@ cudaError_t step_f2_nz(const StepArgsF2 &a, int P, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// FP32 steps: the packed nested kernel (levels in pairs; 32 x 8 tiles of 640 threads up to 30
-// levels, 24 x 8 tiles of 512 threads with 128 registers for 32 levels; measured on the
-// 30-level grid, 32 x 8 tiles at 96 registers beat 24 x 8 at 128, and beat a persistent form
-// that prefetched the next tile's input into the free plane, whose loop spilled registers)
-cudaError_t step_f32(const AdvDev &m, const float *cin, float *cout, int P, const float *src, long long sstride,
-                     float *ebar, long long estride, bool adj, cudaStream_t s)
+
+cudaError_t step_f32_cols(const AdvDev &m, const float *cin, float *cout, int P, const float *src, long long sstride,
+                          float *ebar, long long estride, bool adj, cudaStream_t s)
 {
     StepArgsF2 a;
     const int nzp = m.nz <= 8 ? 4 : m.nz <= 16 ? 8 : m.nz <= 30 ? 15 : 16;
@@ -535,6 +835,56 @@ cudaError_t step_f32(const AdvDev &m, const float *cin, float *cout, int P, cons
     if (nzp == 8) return adj ? step_f2_nz<8, 32, 8, true>(a, P, s) : step_f2_nz<8, 32, 8, false>(a, P, s);
     if (nzp == 15) return adj ? step_f2_nz<15, 32, 8, true>(a, P, s) : step_f2_nz<15, 32, 8, false>(a, P, s);
     return adj ? step_f2_nz<16, 24, 8, true>(a, P, s) : step_f2_nz<16, 24, 8, false>(a, P, s);
+}
+
+constexpr int kZWarps = 12, kZRows = 3;   // 64 x 36 regions of 384 threads with 168 registers
+
+// FP32 steps.  Both forms take whole waves of one CTA per SM; measured per wave on the 30-level
+// grid 32 us for the level-marching form (0.92 us per level and 1 us) and 8.6 us for the
+// column form (0.47 us per pair of levels and 1.5 us).  192 x 192 x 30, 32 columns: 6 waves,
+// 182 us, against 31 waves, 262 us; one column of it 32 against 9 us.
+cudaError_t step_f32(const AdvDev &m, const float *cin, float *cout, int P, const float *src, long long sstride,
+                     float *ebar, long long estride, bool adj, cudaStream_t s)
+{
+    constexpr int TYZ = kZWarps * kZRows - 2 * kHalo;
+    const int sms = num_sms(), nzp = m.nz <= 8 ? 4 : m.nz <= 16 ? 8 : m.nz <= 30 ? 15 : 16;
+    auto waves = [&](int tx, int ty) {
+        return (double)(((long long)((m.nx + tx - 1) / tx) * ((m.ny + ty - 1) / ty) * P + sms - 1) / sms);
+    };
+    if (waves(nzp == 16 ? 24 : 32, 8) * (1.5 + 0.47 * nzp) <= waves(kZTX, TYZ) * (1.0 + 0.92 * (m.nz + 4)))
+        return step_f32_cols(m, cin, cout, P, src, sstride, ebar, estride, adj, s);
+    StepArgsZ a;
+    for (int z = 0; z < kMaxNZ; ++z) {
+        auto kz = [&](int l) { return (l > 0 && l < m.nz) ? (float)(m.kz_h[l] / (m.dz * m.dz)) : 0.f; };
+        a.amp[z] = z < m.nz ? (float)m.amp_h[z] : 0.f;
+        a.ku[z] = kz(z + 1);
+        a.kl[z] = kz(z);
+        a.nkd[z] = -(a.ku[z] + a.kl[z]);
+    }
+    a.cin = cin;
+    a.cout = cout;
+    a.pstride = m.ncells;
+    a.src = src;
+    a.sstride = sstride;
+    a.ebar = ebar;
+    a.estride = estride;
+    a.u = m.u32;
+    a.v = m.v32;
+    a.nx = m.nx;
+    a.ny = m.ny;
+    a.nz = m.nz;
+    a.h = (float)m.dt;
+    const float al[4] = {0.25f * a.h, a.h / 3.f, 0.5f * a.h, a.h};
+    for (int i = 0; i < 4; ++i) {
+        uint32_t w;
+        memcpy(&w, &al[i], 4);
+        a.al[i] = (unsigned long long)w << 32 | w;
+    }
+    a.rdx = (float)(1.0 / m.dx);
+    a.rdy = (float)(1.0 / m.dy);
+    const bool pair = m.nx % 2 == 0 && ((uintptr_t)cin | (uintptr_t)cout) % 8 == 0;
+    if (pair) return adj ? step_z_launch<kZWarps, kZRows, true, true>(a, P, s) : step_z_launch<kZWarps, kZRows, false, true>(a, P, s);
+    return adj ? step_z_launch<kZWarps, kZRows, true, false>(a, P, s) : step_z_launch<kZWarps, kZRows, false, false>(a, P, s);
 }
 
 template <typename R>
