@@ -3,22 +3,11 @@
 // batched RK4 tangent-linear and adjoint steppers, trilinear observation
 // gather / scatter, and the separable exponential prior square root.
 //
-// Stepper design.  One launch advances a batch of sketch columns ("probes")
-// by one RK4 step.  A CTA owns a TX x TY tile of columns (x, y) of one probe,
-// every level, plus a halo of 4 columns on each side: the four RK4 stages are
-// computed on chip, each on a region one column narrower than the last
-// (stage s is valid on the tile grown by 4 - s), so the state is read once
-// and written once per step.  A thread owns one column of the region and
-// keeps its levels in registers (step input, stage input, RK4 accumulator);
-// the horizontal neighbours of a stage input come from one shared-memory
-// plane per level, the vertical ones from the thread's own registers.  The
-// upwind advection of a column reduces to five coefficients (self and the
-// four neighbours) computed once from the face winds and scaled per level;
-// the adjoint uses the transposed coefficients, so the same kernel steps
-// both directions.  For a linear autonomous system the RK4 step is
-// c+ = P(hA) c + h Q(hA) s, and its adjoint gives the source adjoint
-// h Q(hA^T) lam = h/6 (lam + 2 u1 + 2 u2 + u3) from the adjoint stage inputs
-// u1..u3, accumulated at level 0 for the emission blocks.
+// The upwind advection of a column reduces to five coefficients (self and the four neighbours)
+// computed from the face winds and scaled per level; the adjoint uses the transposed ones, so
+// the same kernels step both directions.  For a linear autonomous system the RK4 step is
+// c+ = P(hA) c + h Q(hA) s, and its adjoint gives the source adjoint h Q(hA^T) lam, added at
+// level 0 of the emission blocks.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -34,120 +23,82 @@ constexpr int kHalo = 4;
 
 constexpr int kMaxNZ = 32;
 
-template <typename R>
-struct StepArgs {
-    R amp[kMaxNZ];        // level scaling of the winds (0 beyond nz)
-    R kzs[kMaxNZ + 1];    // Kz / dz^2 on face l-1/2 (0 on the bottom, the top and beyond)
-    const R *cin;
-    R *cout;
+// FP64 stepper: one launch per RK4 stage, one cell per thread.  The stages are the nested
+// (Horner) form w_{s+1} = c + a_s (A w_s + s), a = h/4, h/3, h/2, h, w_0 = c, w_4 = c+ (equal to
+// the classical stages for a linear autonomous tendency; see the FP32 stepper), ten FP64
+// operations a cell.  Bound: FP64 issue, one warp instruction per 64 cycles and sub-partition,
+// so nothing is computed twice (a step fused in one kernel computes 3.1 times the cells on the
+// 16 x 2 tiles that fit) and every cell is a thread (4.6 us of issue per stage on 96 x 96 x 30);
+// the re-read fields come from L2, the column coefficients from a table.  A launch is a
+// programmatic dependent of the one before, so that its start overlaps that one's end.
+// Measured: riot_outer_begin of 96 x 96 x 30 and 60 steps 16.86 -> 3.78 ms (134 -> 27 us a step).
+struct StageArgs {
+    double amp[kMaxNZ], ku[kMaxNZ], kl[kMaxNZ], nkd[kMaxNZ];
+    const double *w, *c;
+    double *out;
     long long pstride;    // cells per probe
-    const R *src;         // surface source of this step's block (TL), per probe at sstride
+    const double *cf;     // [5][ny][nx] self, east, west, north, south
+    const double *src;    // surface source of this step's block (TL), per probe at sstride
     long long sstride;
-    R *ebar;              // source adjoint of this step's block (AD), per probe at estride
+    double *ebar;         // source adjoint of this step's block (last stage of AD), per probe at estride
     long long estride;
-    const R *u, *v;
     int nx, ny, nz;
-    R h, rdx, rdy;
+    double al;
 };
 
-template <typename R, int NZ, int TX, int TY, bool ADJ>
-__global__ void __launch_bounds__((TX + 2 * kHalo) * (TY + 2 * kHalo), 1) adv_step_kernel(StepArgs<R> a)
+constexpr int kStageBlock = 128;
+
+__global__ void __launch_bounds__(kStageBlock) adv_stage_kernel(const __grid_constant__ StageArgs a)
 {
-    constexpr int RX = TX + 2 * kHalo, RY = TY + 2 * kHalo, PL = RX * RY;
-    extern __shared__ __align__(16) unsigned char adv_smem[];
-    // two [NZ][RY][RX] planes of stage inputs, used alternately: one barrier per stage
-    R *S0 = reinterpret_cast<R *>(adv_smem);
-    const int tid = threadIdx.x;
-    const int rx = tid % RX, ry = tid / RX;
-    const int nx = a.nx, ny = a.ny;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-    int gx = (x0 - kHalo + rx) % nx;
-    if (gx < 0) gx += nx;
-    const int gy = y0 - kHalo + ry;
-    const bool valid = gy >= 0 && gy < ny;
-    const size_t plane = (size_t)nx * ny;
-    const size_t col = valid ? (size_t)gy * nx + gx : 0;
-    // advection coefficients of this column at amplitude 1 (1/s)
-    R c0 = 0, cE = 0, cW = 0, cN = 0, cS = 0;
-    if (valid) {
-        const R uL = a.u[col], uR = a.u[(size_t)gy * nx + (gx + 1 == nx ? 0 : gx + 1)];
-        const R vS = a.v[col], vN = a.v[col + nx];
-        const R z0 = R(0);
-        const R uLp = uL > z0 ? uL : z0, uLm = uL < z0 ? uL : z0;
-        const R uRp = uR > z0 ? uR : z0, uRm = uR < z0 ? uR : z0;
-        const R vSp = vS > z0 ? vS : z0, vSm = vS < z0 ? vS : z0;
-        const R vNp = vN > z0 ? vN : z0, vNm = vN < z0 ? vN : z0;
-        c0 = (uLm - uRp) * a.rdx + (vSm - vNp) * a.rdy;
-        if (!ADJ) {
-            cE = -uRm * a.rdx;
-            cW = uLp * a.rdx;
-            cN = -vNm * a.rdy;
-            cS = vSp * a.rdy;
-        } else {
-            cE = uRp * a.rdx;
-            cW = -uLm * a.rdx;
-            cN = vNp * a.rdy;
-            cS = -vSm * a.rdy;
-        }
+    const int plane = a.nx * a.ny, col = blockIdx.x * kStageBlock + threadIdx.x, z = blockIdx.y;
+    if (col >= plane) {
+        cudaGridDependencySynchronize();
+        return;
     }
-    const size_t pb = (size_t)blockIdx.z * a.pstride;
-    R c[NZ], w[NZ], acc[NZ];
+    const int y = col / a.nx, x = col - y * a.nx;
+    const int cE = x + 1 == a.nx ? col + 1 - a.nx : col + 1, cW = x == 0 ? col + a.nx - 1 : col - 1;
+    const int cN = y + 1 == a.ny ? col : col + a.nx, cS = y == 0 ? col : col - a.nx;   // walls: coefficient 0
+    double k[5];
 #pragma unroll
-    for (int z = 0; z < NZ; ++z) {
-        c[z] = (valid && z < a.nz) ? a.cin[pb + z * plane + col] : R(0);
-        w[z] = c[z];
-        acc[z] = R(0);
+    for (int i = 0; i < 5; ++i) k[i] = a.cf[(size_t)i * plane + col];
+    cudaGridDependencySynchronize();
+    const size_t at = (size_t)blockIdx.z * a.pstride + (size_t)z * plane;
+    const double *w = a.w + at;
+    const double wo = w[col], up = z + 1 < a.nz ? w[plane + col] : 0.0, dn = z > 0 ? w[col - plane] : 0.0;
+    const double wE = w[cE], wW = w[cW], wN = w[cN], wS = w[cS], c = a.c[at + col];
+    cudaTriggerProgrammaticLaunchCompletion();
+    double q = k[0] * wo;
+    q = fma(k[1], wE, q);
+    q = fma(k[2], wW, q);
+    q = fma(k[3], wN, q);
+    q = fma(k[4], wS, q);
+    q *= a.amp[z];
+    q = fma(a.ku[z], up, q);
+    q = fma(a.kl[z], dn, q);
+    q = fma(a.nkd[z], wo, q);
+    if (z == 0) {
+        if (a.src) q += a.src[(size_t)blockIdx.z * a.sstride + col];
+        if (a.ebar) a.ebar[(size_t)blockIdx.z * a.estride + col] += a.al * wo;   // al = h in the last stage
     }
-    R s0 = R(0);
-    if (!ADJ && valid && a.src) s0 = a.src[(size_t)blockIdx.z * a.sstride + col];
-    const R h = a.h, h2 = R(0.5) * a.h, h3 = a.h / R(3), h6 = a.h / R(6);
-    R e0 = R(0);
+    a.out[at + col] = fma(a.al, q, c);
+}
+
+// Column coefficients of both directions: cf[0] tangent linear, cf[1] adjoint, [5][ny][nx] each.
+__global__ void adv_coef_kernel(const double *u, const double *v, int nx, int ny, double rdx, double rdy, double *cf)
+{
+    const int plane = nx * ny, col = blockIdx.x * blockDim.x + threadIdx.x;
+    if (col >= plane) return;
+    const int x = col % nx;
+    const double uL = u[col], uR = u[x + 1 == nx ? col + 1 - nx : col + 1], vS = v[col], vN = v[col + nx];
+    const double uLp = fmax(uL, 0.0), uLm = fmin(uL, 0.0), uRp = fmax(uR, 0.0), uRm = fmin(uR, 0.0);
+    const double vSp = fmax(vS, 0.0), vSm = fmin(vS, 0.0), vNp = fmax(vN, 0.0), vNm = fmin(vN, 0.0);
+    const double c0 = (uLm - uRp) * rdx + (vSm - vNp) * rdy;
+    const double tl[5] = {c0, -uRm * rdx, uLp * rdx, -vNm * rdy, vSp * rdy};
+    const double ad[5] = {c0, uRp * rdx, -uLm * rdx, vNp * rdy, -vSm * rdy};
 #pragma unroll
-    for (int st = 1; st <= 4; ++st) {
-        R *S = S0 + (st & 1) * NZ * PL;
-        // the stage input is read on the region of this stage grown by one column;
-        // rows beyond the walls publish their zeros (their coefficients are 0, but
-        // a stale value times 0 would not be)
-        const bool pub = rx >= st - 1 && rx < RX - st + 1 && ry >= st - 1 && ry < RY - st + 1;
-        if (pub) {
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) S[z * PL + ry * RX + rx] = w[z];
-        }
-        if (ADJ) e0 += (st == 1 || st == 4) ? w[0] : R(2) * w[0];
-        __syncthreads();
-        const bool act = valid && rx >= st && rx < RX - st && ry >= st && ry < RY - st;
-        if (act) {
-            R wm = R(0);
-#pragma unroll
-            for (int z = 0; z < NZ; ++z) {
-                const R wz = w[z];
-                const R wp = (z + 1 < NZ) ? w[z + 1] : R(0);
-                const R *Sz = S + z * PL + ry * RX + rx;
-                const R hor = c0 * wz + cE * Sz[1] + cW * Sz[-1] + cN * Sz[RX] + cS * Sz[-RX];
-                R k = a.amp[z] * hor + a.kzs[z + 1] * (wp - wz) - a.kzs[z] * (wz - wm);
-                if (!ADJ && z == 0) k += s0;
-                if (st == 1) {
-                    acc[z] = c[z] + h6 * k;
-                    w[z] = c[z] + h2 * k;
-                } else if (st == 2) {
-                    acc[z] += h3 * k;
-                    w[z] = c[z] + h2 * k;
-                } else if (st == 3) {
-                    acc[z] += h3 * k;
-                    w[z] = c[z] + h * k;
-                } else {
-                    acc[z] += h6 * k;
-                }
-                wm = wz;
-            }
-        }
-    }
-    const int ix = rx - kHalo, iy = ry - kHalo;
-    if (valid && ix >= 0 && ix < TX && iy >= 0 && iy < TY && x0 + ix < nx) {
-#pragma unroll
-        for (int z = 0; z < NZ; ++z)
-            if (z < a.nz) a.cout[pb + z * plane + col] = acc[z];
-        if (ADJ && a.ebar) a.ebar[(size_t)blockIdx.z * a.estride + col] += h6 * e0;
+    for (int i = 0; i < 5; ++i) {
+        cf[(size_t)i * plane + col] = tl[i];
+        cf[(size_t)(5 + i) * plane + col] = ad[i];
     }
 }
 
@@ -445,7 +396,8 @@ __global__ void __launch_bounds__(32 * NW) adv_step_z_kernel(const __grid_consta
 // combined by packed FP32x2 instructions, one instruction for two levels; the shared planes
 // hold the pairs, so a horizontal neighbour fetch is one 64-bit load for two levels.  (Pairs
 // (p, p + NZP), whose vertical neighbours are whole pairs, measured slower: the renamed
-// stage inputs cost registers.)  Tiles and halo as in adv_step_kernel.
+// stage inputs cost registers.)  A CTA owns a TX x TY tile of one
+// probe plus a halo of 4 columns on each side, each stage on a region one column narrower.
 struct StepArgsF2 {
     float2 amp2[16];   // (amp of level 2p, of level 2p + 1); 0 beyond nz
     float2 ku2[16];    // Kz / dz^2 on the face above each level of the pair
@@ -510,6 +462,7 @@ __global__ void __maxnreg__(regs_for((TX + 2 * kHalo) * (TY + 2 * kHalo))) adv_s
     const float2 C0 = make_float2(c0, c0), CE = make_float2(cE, cE), CW = make_float2(cW, cW);
     const float2 CN = make_float2(cN, cN), CS = make_float2(cS, cS);
     const size_t pb = (size_t)blockIdx.z * a.pstride;
+    cudaGridDependencySynchronize();
     float2 c[NZP], w[NZP];
 #pragma unroll
     for (int p = 0; p < NZP; ++p) {
@@ -531,6 +484,7 @@ __global__ void __maxnreg__(regs_for((TX + 2 * kHalo) * (TY + 2 * kHalo))) adv_s
             for (int p = 0; p < NZP; ++p) S[p * PL + ry * RX + rx] = w[p];
         }
         if (ADJ && st == 3) e0 = w[0].x;
+        if (st == 3) cudaTriggerProgrammaticLaunchCompletion();
         __syncthreads();
         if (valid && rx > st && rx < RX - st - 1 && ry > st && ry < RY - st - 1) {
             const float al = (st == 0) ? 0.25f * a.h : (st == 1) ? a.h / 3.f : (st == 2) ? 0.5f * a.h : a.h;
@@ -573,41 +527,62 @@ template <typename R>
 __global__ void obs_gather_kernel(const R *c, long long pstride, int o0, int no, const int *cell, const R *w,
                                   const R *rinv, R *r, long long rstride)
 {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = blockIdx.x * blockDim.x + threadIdx.x, oo = o0 + (o < no ? o : 0);
+    R wq[8];
+    int cq[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        wq[q] = w[8 * oo + q];
+        cq[q] = cell[8 * oo + q];
+    }
+    const R ri = rinv[oo];
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
     if (o >= no) return;
-    const int oo = o0 + o;
     const R *cp = c + (size_t)blockIdx.y * pstride;
     R acc = R(0);
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc += w[8 * oo + q] * cp[cell[8 * oo + q]];
-    r[(size_t)blockIdx.y * rstride + oo] = rinv[oo] * acc;
+    for (int q = 0; q < 8; ++q) acc += wq[q] * cp[cq[q]];
+    r[(size_t)blockIdx.y * rstride + oo] = ri * acc;
 }
 
 __global__ void obs_innov_kernel(const double *c, int o0, int no, const int *cell, const double *w,
                                  const double *y, const double *rinv, double *d, double *jo)
 {
     const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= no) return;
-    const int oo = o0 + o;
-    double acc = 0.0;
+    double j = 0.0;
+    if (o < no) {
+        const int oo = o0 + o;
+        double acc = 0.0;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) acc += w[8 * oo + q] * c[cell[8 * oo + q]];
-    const double dd = acc - y[oo];
-    d[oo] = dd;
-    atomicAdd(jo, 0.5 * dd * dd * rinv[oo]);
+        for (int q = 0; q < 8; ++q) acc += w[8 * oo + q] * c[cell[8 * oo + q]];
+        const double dd = acc - y[oo];
+        d[oo] = dd;
+        j = 0.5 * dd * dd * rinv[oo];
+    }
+    for (int off = 16; off > 0; off >>= 1) j += __shfl_down_sync(0xffffffffu, j, off);
+    if ((threadIdx.x & 31) == 0 && j != 0.0) atomicAdd(jo, j);
 }
 
 template <typename R>
 __global__ void obs_scatter_kernel(R *lam, long long pstride, int o0, int no, const int *cell, const R *w,
                                    const R *r, long long rstride)
 {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
+    const int o = blockIdx.x * blockDim.x + threadIdx.x, oo = o0 + (o < no ? o : 0);
+    R wq[8];
+    int cq[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        wq[q] = w[8 * oo + q];
+        cq[q] = cell[8 * oo + q];
+    }
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
     if (o >= no) return;
-    const int oo = o0 + o;
     R *lp = lam + (size_t)blockIdx.y * pstride;
     const R rv = r[(size_t)blockIdx.y * rstride + oo];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) atomicAdd(&lp[cell[8 * oo + q]], w[8 * oo + q] * rv);
+    for (int q = 0; q < 8; ++q) atomicAdd(&lp[cq[q]], wq[q] * rv);
 }
 
 // Batched row-major GEMM C_f = alpha A_f B_f (M x K times K x N); the batch
@@ -675,6 +650,29 @@ __global__ void __launch_bounds__(256) bgemm_kernel(BGArgs<R> g)
     }
 }
 
+// The same with one output per thread on 16 x 16 tiles, for few FP64 fields: a 64 x 64 tile is 95
+// us of one SM's FP64 issue at K = 96 whatever the grid, a 16 x 16 tile 6 us.
+__global__ void __launch_bounds__(256) bgemm16_kernel(BGArgs<double> g)
+{
+    __shared__ double As[16][17], Bs[16][17];
+    const int f = blockIdx.z;
+    const double *A = g.A + (f / g.inner) * g.aso + (f % g.inner) * g.asi;
+    const double *B = g.B + (f / g.inner) * g.bso + (f % g.inner) * g.bsi;
+    double *C = g.C + (f / g.inner) * g.cso + (f % g.inner) * g.csi;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int mm = blockIdx.y * 16 + ty, nn = blockIdx.x * 16 + tx;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < g.K; k0 += 16) {
+        As[ty][tx] = (mm < g.M && k0 + tx < g.K) ? A[(size_t)mm * g.lda + k0 + tx] : 0.0;
+        Bs[ty][tx] = (k0 + ty < g.K && nn < g.N) ? B[(size_t)(k0 + ty) * g.ldb + nn] : 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < 16; ++kk) acc = fma(As[ty][kk], Bs[kk][tx], acc);
+        __syncthreads();
+    }
+    if (mm < g.M && nn < g.N) C[(size_t)mm * g.ldc + nn] = g.alpha * acc;
+}
+
 // out[j*ldo + i] = in[j*ldi + i] * s[i] (+ add[j*lda + i])
 template <typename R>
 __global__ void colscale_kernel(const R *in, long long ldi, const R *s, R *out, long long ldo, int n, int ncols)
@@ -734,36 +732,26 @@ struct Tab<double> {
     static const double *Es(const AdvDev &m) { return m.Es64; }
 };
 
-// Tile shape per precision: FP32 keeps 3 x NZ floats per thread with 480
-// threads; FP64 needs twice the registers per level, so its tiles are smaller.
-template <typename R>
-struct TileShape;
-template <>
-struct TileShape<float> {
-    static constexpr int TX = 32, TY = 4;
-};
-template <>
-struct TileShape<double> {
-    static constexpr int TX = 16, TY = 2;
-};
-
-template <typename R, int NZ, bool ADJ>
-cudaError_t step_nz(const StepArgs<R> &a, int P, cudaStream_t s)
+// Small grids spend their time between kernels: a step of 37 x 23 x 11 with 16 probes and its
+// observation kernel took 12 us, 6.8 us since each starts during the one before (products of 48
+// steps 1.14 -> 0.65 ms).
+// Launch as a programmatic dependent of the kernel before it in the stream (which it waits for
+// itself, by cudaGridDependencySynchronize, before it reads or writes what that one may touch).
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A &...args)
 {
-    constexpr int TX = TileShape<R>::TX, TY = TileShape<R>::TY;
-    constexpr int RX = TX + 2 * kHalo, RY = TY + 2 * kHalo;
-    const size_t smem = sizeof(R) * 2 * (size_t)NZ * RX * RY;
-    auto kern = adv_step_kernel<R, NZ, TX, TY, ADJ>;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
-    dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, P);
-    kern<<<grid, RX * RY, smem, s>>>(a);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
     count_launch();
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 template <int NW, int RW, bool ADJ, bool PAIR>
@@ -797,9 +785,7 @@ cudaError_t step_f2_nz(const StepArgsF2 &a, int P, cudaStream_t s)
         attr_done = true;
     }
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, P);
-    kern<<<grid, RX * RY, smem, s>>>(a);
-    count_launch();
-    return cudaGetLastError();
+    return launch_after(kern, grid, RX * RY, smem, s, a);
 }
 
 
@@ -887,33 +873,58 @@ cudaError_t step_f32(const AdvDev &m, const float *cin, float *cout, int P, cons
     return adj ? step_z_launch<kZWarps, kZRows, true, false>(a, P, s) : step_z_launch<kZWarps, kZRows, false, false>(a, P, s);
 }
 
-template <typename R>
-cudaError_t step(const AdvDev &m, const R *cin, R *cout, int P, const R *src, long long sstride, R *ebar,
-                 long long estride, bool adj, cudaStream_t s)
+// One step of P probes in FP64: cA -> cB, cX scratch of the same size.
+cudaError_t step_f64(const AdvDev &m, const double *cA, double *cB, double *cX, int P, const double *src,
+                     long long sstride, double *ebar, long long estride, bool adj, cudaStream_t s)
 {
-    if constexpr (sizeof(R) == sizeof(float)) return step_f32(m, cin, cout, P, src, sstride, ebar, estride, adj, s);
-    StepArgs<R> a;
-    a.cin = cin;
-    a.cout = cout;
+    StageArgs a;
+    for (int l = 0; l < kMaxNZ; ++l) {
+        auto kz = [&](int f) { return (f > 0 && f < m.nz) ? m.kz_h[f] / (m.dz * m.dz) : 0.0; };
+        a.amp[l] = l < m.nz ? m.amp_h[l] : 0.0;
+        a.ku[l] = kz(l + 1);
+        a.kl[l] = kz(l);
+        a.nkd[l] = -(a.ku[l] + a.kl[l]);
+    }
     a.pstride = m.ncells;
+    a.cf = m.cf64 + (adj ? (size_t)5 * m.nx * m.ny : 0);
     a.src = src;
     a.sstride = sstride;
-    a.ebar = ebar;
     a.estride = estride;
-    a.u = Tab<R>::u(m);
-    a.v = Tab<R>::v(m);
-    for (int l = 0; l < kMaxNZ; ++l) a.amp[l] = l < m.nz ? (R)m.amp_h[l] : R(0);
-    for (int l = 0; l <= kMaxNZ; ++l)
-        a.kzs[l] = (l > 0 && l < m.nz) ? (R)(m.kz_h[l] / (m.dz * m.dz)) : R(0);
     a.nx = m.nx;
     a.ny = m.ny;
     a.nz = m.nz;
-    a.h = (R)m.dt;
-    a.rdx = (R)(1.0 / m.dx);
-    a.rdy = (R)(1.0 / m.dy);
-    if (m.nz <= 8) return adj ? step_nz<R, 8, true>(a, P, s) : step_nz<R, 8, false>(a, P, s);
-    if (m.nz <= 16) return adj ? step_nz<R, 16, true>(a, P, s) : step_nz<R, 16, false>(a, P, s);
-    return adj ? step_nz<R, 32, true>(a, P, s) : step_nz<R, 32, false>(a, P, s);
+    a.c = cA;
+    const double al[4] = {0.25 * m.dt, m.dt / 3.0, 0.5 * m.dt, m.dt};
+    const double *in[4] = {cA, cX, cB, cX};
+    double *out[4] = {cX, cB, cX, cB};
+    const dim3 grid((m.nx * m.ny + kStageBlock - 1) / kStageBlock, m.nz, P);
+    for (int st = 0; st < 4; ++st) {
+        a.w = in[st];
+        a.out = out[st];
+        a.al = al[st];
+        a.ebar = adj && st == 3 ? ebar : nullptr;
+        const cudaError_t e = launch_after(adv_stage_kernel, grid, kStageBlock, 0, s, a);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <typename R>
+cudaError_t step(const AdvDev &m, const R *cin, R *cout, R *scratch, int P, const R *src, long long sstride, R *ebar,
+                 long long estride, bool adj, cudaStream_t s)
+{
+    if constexpr (sizeof(R) == sizeof(float)) return step_f32(m, cin, cout, P, src, sstride, ebar, estride, adj, s);
+    else return step_f64(m, cin, cout, scratch, P, src, sstride, ebar, estride, adj, s);
+}
+
+// The batch workspace as two fields of P probes (and the scratch field of FP64 steps).
+template <typename R>
+void batch_fields(const AdvDev &m, int P, R **cA, R **cB, R **cX)
+{
+    const size_t cells = (size_t)P * m.ncells;
+    *cA = (R *)m.fields;
+    *cB = *cA + cells;
+    *cX = 3 * cells * sizeof(R) <= m.fields_bytes ? *cB + cells : (R *)m.c64X;   // FP64: c64X holds one probe
 }
 
 template <typename R>
@@ -922,9 +933,8 @@ cudaError_t gather(const AdvDev &m, const R *c, int P, int t, R *r, long long rs
     const int o0 = m.optr_h[t], no = m.optr_h[t + 1] - o0;
     if (no <= 0) return cudaSuccess;
     dim3 grid(blocks_for(no, 128), P);
-    obs_gather_kernel<R><<<grid, 128, 0, s>>>(c, m.ncells, o0, no, m.cell, Tab<R>::w(m), Tab<R>::rinv(m), r, rstride);
-    count_launch();
-    return cudaGetLastError();
+    return launch_after(obs_gather_kernel<R>, grid, 128, 0, s, c, (long long)m.ncells, o0, no, m.cell, Tab<R>::w(m),
+                        Tab<R>::rinv(m), r, rstride);
 }
 
 template <typename R>
@@ -933,15 +943,22 @@ cudaError_t scatter(const AdvDev &m, R *lam, int P, int t, const R *r, long long
     const int o0 = m.optr_h[t], no = m.optr_h[t + 1] - o0;
     if (no <= 0) return cudaSuccess;
     dim3 grid(blocks_for(no, 128), P);
-    obs_scatter_kernel<R><<<grid, 128, 0, s>>>(lam, m.ncells, o0, no, m.cell, Tab<R>::w(m), r, rstride);
-    count_launch();
-    return cudaGetLastError();
+    return launch_after(obs_scatter_kernel<R>, grid, 128, 0, s, lam, (long long)m.ncells, o0, no, m.cell, Tab<R>::w(m), r,
+                        rstride);
 }
 
 template <typename R>
 cudaError_t bgemm(const BGArgs<R> &g, int batch, cudaStream_t s)
 {
     dim3 grid((g.N + 63) / 64, (g.M + 63) / 64, batch);
+    if constexpr (sizeof(R) == sizeof(double)) {
+        if ((long long)grid.x * grid.y * batch < 4 * num_sms()) {
+            grid = dim3((g.N + 15) / 16, (g.M + 15) / 16, batch);
+            bgemm16_kernel<<<grid, 256, 0, s>>>(g);
+            count_launch();
+            return cudaGetLastError();
+        }
+    }
     bgemm_kernel<R><<<grid, 256, 0, s>>>(g);
     count_launch();
     return cudaGetLastError();
@@ -1014,8 +1031,9 @@ cudaError_t hvp_batch(const AdvDev &m, const R *W, R *Y, long long ld, int P, in
 {
     cudaError_t e;
     const long long n = m.n, nyx = (long long)m.ny * m.nx;
-    R *cA = (R *)m.cA, *cB = (R *)m.cB, *src = (R *)m.src, *ebar = (R *)m.ebar, *tmp = (R *)m.tmp;
+    R *cA, *cB, *cX, *src = (R *)m.src, *ebar = (R *)m.ebar, *tmp = (R *)m.tmp;
     const size_t cells = (size_t)P * m.ncells;
+    batch_fields(m, P, &cA, &cB, &cX);
 #define ADV_TRY(x)                          \
     do {                                    \
         if ((e = (x)) != cudaSuccess) return e; \
@@ -1027,7 +1045,7 @@ cudaError_t hvp_batch(const AdvDev &m, const R *W, R *Y, long long ld, int P, in
     ADV_TRY(cudaMemsetAsync(cA, 0, cells * sizeof(R), s));
     for (int t = 0; t < m.T; ++t) {
         const int b = (int)(((long long)t * m.nb) / m.T);
-        ADV_TRY(step<R>(m, cA, cB, P, src + b * nyx, n, nullptr, 0, false, s));
+        ADV_TRY(step<R>(m, cA, cB, cX, P, src + b * nyx, n, nullptr, 0, false, s));
         R *sw = cA;
         cA = cB;
         cB = sw;
@@ -1039,7 +1057,7 @@ cudaError_t hvp_batch(const AdvDev &m, const R *W, R *Y, long long ld, int P, in
     for (int t = m.T - 1; t >= 0; --t) {
         ADV_TRY(scatter<R>(m, cA, P, t + 1, r, m.p, s));
         const int b = (int)(((long long)t * m.nb) / m.T);
-        ADV_TRY(step<R>(m, cA, cB, P, nullptr, 0, ebar + b * nyx, n, true, s));
+        ADV_TRY(step<R>(m, cA, cB, cX, P, nullptr, 0, ebar + b * nyx, n, true, s));
         R *sw = cA;
         cA = cB;
         cB = sw;
@@ -1065,14 +1083,15 @@ cudaError_t tl_batch(const AdvDev &m, const R *W, long long ldw, int P, R *r, cu
 {
     cudaError_t e;
     const long long n = m.n, nyx = (long long)m.ny * m.nx;
-    R *cA = (R *)m.cA, *cB = (R *)m.cB, *src = (R *)m.src, *tmp = (R *)m.tmp;
+    R *cA, *cB, *cX, *src = (R *)m.src, *tmp = (R *)m.tmp;
     const size_t cells = (size_t)P * m.ncells;
+    batch_fields(m, P, &cA, &cB, &cX);
     if ((e = sep_apply<R>(m, W, ldw, src, n, P, tmp, s)) != cudaSuccess) return e;
     if ((e = colscale<R>(src, n, Tab<R>::Es(m), src, n, (int)n, P, s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(cA, 0, cells * sizeof(R), s)) != cudaSuccess) return e;
     for (int t = 0; t < m.T; ++t) {
         const int b = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<R>(m, cA, cB, P, src + b * nyx, n, nullptr, 0, false, s)) != cudaSuccess) return e;
+        if ((e = step<R>(m, cA, cB, cX, P, src + b * nyx, n, nullptr, 0, false, s)) != cudaSuccess) return e;
         R *sw = cA;
         cA = cB;
         cB = sw;
@@ -1086,14 +1105,15 @@ cudaError_t ad_batch(const AdvDev &m, const R *f, int P, R *Z, long long ldz, cu
 {
     cudaError_t e;
     const long long n = m.n, nyx = (long long)m.ny * m.nx;
-    R *cA = (R *)m.cA, *cB = (R *)m.cB, *ebar = (R *)m.ebar, *tmp = (R *)m.tmp;
+    R *cA, *cB, *cX, *ebar = (R *)m.ebar, *tmp = (R *)m.tmp;
     const size_t cells = (size_t)P * m.ncells;
+    batch_fields(m, P, &cA, &cB, &cX);
     if ((e = cudaMemsetAsync(cA, 0, cells * sizeof(R), s)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(ebar, 0, (size_t)P * n * sizeof(R), s)) != cudaSuccess) return e;
     for (int t = m.T - 1; t >= 0; --t) {
         if ((e = scatter<R>(m, cA, P, t + 1, f, m.p, s)) != cudaSuccess) return e;
         const int b = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<R>(m, cA, cB, P, nullptr, 0, ebar + b * nyx, n, true, s)) != cudaSuccess) return e;
+        if ((e = step<R>(m, cA, cB, cX, P, nullptr, 0, ebar + b * nyx, n, true, s)) != cudaSuccess) return e;
         R *sw = cA;
         cA = cB;
         cB = sw;
@@ -1103,6 +1123,14 @@ cudaError_t ad_batch(const AdvDev &m, const R *f, int P, R *Z, long long ldz, cu
 }
 
 }  // namespace
+
+cudaError_t adv_coefs(const AdvDev &m, cudaStream_t s)
+{
+    count_launch();
+    adv_coef_kernel<<<blocks_for((size_t)m.nx * m.ny, 256), 256, 0, s>>>(m.u64, m.v64, m.nx, m.ny, 1.0 / m.dx, 1.0 / m.dy,
+                                                                          m.cf64);
+    return cudaGetLastError();
+}
 
 cudaError_t adv_tl(const AdvDev &m, const double *W, int64_t ld, int ncols, double *r, cudaStream_t s)
 {
@@ -1134,7 +1162,7 @@ cudaError_t adv_ad_obs(const AdvDev &m, const double *f, double *z, cudaStream_t
     for (int t = m.T - 1; t >= 0; --t) {
         if ((e = scatter<double>(m, cA, 1, t + 1, f, m.p, s)) != cudaSuccess) return e;
         const int bk = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<double>(m, cA, cB, 1, nullptr, 0, m.ebar64 + bk * nyx, n, true, s)) != cudaSuccess) return e;
+        if ((e = step<double>(m, cA, cB, m.c64X, 1, nullptr, 0, m.ebar64 + bk * nyx, n, true, s)) != cudaSuccess) return e;
         double *sw = cA;
         cA = cB;
         cB = sw;
@@ -1172,7 +1200,7 @@ cudaError_t adv_outer(const AdvDev &m, const double *x, double *d, double *jo, d
     if ((e = cudaMemsetAsync(cA, 0, (size_t)m.ncells * sizeof(double), s)) != cudaSuccess) return e;
     for (int t = 0; t < m.T; ++t) {
         const int bk = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<double>(m, cA, cB, 1, m.Es64 + bk * nyx, 0, nullptr, 0, false, s)) != cudaSuccess) return e;
+        if ((e = step<double>(m, cA, cB, m.c64X, 1, m.Es64 + bk * nyx, 0, nullptr, 0, false, s)) != cudaSuccess) return e;
         double *sw = cA;
         cA = cB;
         cB = sw;
@@ -1192,7 +1220,7 @@ cudaError_t adv_outer(const AdvDev &m, const double *x, double *d, double *jo, d
     for (int t = m.T - 1; t >= 0; --t) {
         if ((e = scatter<double>(m, cA, 1, t + 1, rd, m.p, s)) != cudaSuccess) return e;
         const int bk = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<double>(m, cA, cB, 1, nullptr, 0, m.ebar64 + bk * nyx, n, true, s)) != cudaSuccess) return e;
+        if ((e = step<double>(m, cA, cB, m.c64X, 1, nullptr, 0, m.ebar64 + bk * nyx, n, true, s)) != cudaSuccess) return e;
         double *sw = cA;
         cA = cB;
         cB = sw;
@@ -1212,7 +1240,7 @@ cudaError_t adv_tl_obs(const AdvDev &m, const double *w, double *r, cudaStream_t
     if ((e = cudaMemsetAsync(cA, 0, (size_t)m.ncells * sizeof(double), s)) != cudaSuccess) return e;
     for (int t = 0; t < m.T; ++t) {
         const int bk = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<double>(m, cA, cB, 1, src + bk * nyx, n, nullptr, 0, false, s)) != cudaSuccess) return e;
+        if ((e = step<double>(m, cA, cB, m.c64X, 1, src + bk * nyx, n, nullptr, 0, false, s)) != cudaSuccess) return e;
         double *sw = cA;
         cA = cB;
         cB = sw;
@@ -1244,7 +1272,7 @@ cudaError_t adv_forecast(const AdvDev &m, const double *x, int steps, double *c_
     if ((e = cudaMemsetAsync(cA, 0, (size_t)m.ncells * sizeof(double), s)) != cudaSuccess) return e;
     for (int t = 0; t < steps; ++t) {
         const int bk = (int)(((long long)t * m.nb) / m.T);
-        if ((e = step<double>(m, cA, cB, 1, m.Es64 + bk * nyx, 0, nullptr, 0, false, s)) != cudaSuccess) return e;
+        if ((e = step<double>(m, cA, cB, m.c64X, 1, m.Es64 + bk * nyx, 0, nullptr, 0, false, s)) != cudaSuccess) return e;
         double *sw = cA;
         cA = cB;
         cB = sw;

@@ -787,24 +787,29 @@ riot_status setup_advdiff(riot_ctx *ctx, const riot_model_desc *model, const rio
     const bool fp64 = ctx->prec == RIOT_PREC_FP64;
     const size_t rs = real_size(ctx);
     a.Pmax64 = ctx->kmax < 64 ? ctx->kmax : 64;
-    a.Pmax = fp64 ? a.Pmax64 : (ctx->kmax < 128 ? ctx->kmax : 128);
-    const size_t P = (size_t)a.Pmax;
-    // bytes per cell (per control) of the batch workspace: at least one FP64 probe
+    const int Pb = fp64 ? a.Pmax64 : (ctx->kmax < 128 ? ctx->kmax : 128);
+    const size_t P = (size_t)Pb;
+    // bytes per cell (per control) of the batch workspace: at least one FP64 probe.  Its two
+    // fields of Pb probes serve FP64 steps as three fields of two thirds as many.
     const size_t wsb = P * rs > sizeof(double) ? P * rs : sizeof(double);
-    a.Pws64 = (int)(wsb / sizeof(double));
-    char *cA = nullptr, *cB = nullptr, *src = nullptr, *ebar = nullptr, *tmp = nullptr;
-    TRY(dalloc(ctx, &cA, wsb * ncells));
-    TRY(dalloc(ctx, &cB, wsb * ncells));
+    const int third = (int)(2 * wsb / (3 * sizeof(double)));
+    a.Pws64 = third > 1 ? third : 1;
+    a.Pmax = fp64 ? a.Pws64 : Pb;
+    a.fields_bytes = 2 * wsb * ncells;
+    char *fields = nullptr, *src = nullptr, *ebar = nullptr, *tmp = nullptr;
+    TRY(dalloc(ctx, &fields, a.fields_bytes));
     TRY(dalloc(ctx, &src, wsb * n));
     TRY(dalloc(ctx, &ebar, wsb * n));
     TRY(dalloc(ctx, &tmp, wsb * n));
-    a.cA = cA;
-    a.cB = cB;
+    a.fields = fields;
     a.src = src;
     a.ebar = ebar;
     a.tmp = tmp;
     TRY(dalloc(ctx, &a.c64A, ncells));
     TRY(dalloc(ctx, &a.c64B, ncells));
+    TRY(dalloc(ctx, &a.c64X, ncells));
+    TRY(dalloc(ctx, &a.cf64, (size_t)10 * nyx));
+    CU(adv_coefs(a, ctx->s));
     TRY(dalloc(ctx, &a.ebar64, n));
     TRY(dalloc(ctx, &a.tmp64, (size_t)a.Pmax64 * n));
     TRY(dalloc(ctx, &a.Es64, n));

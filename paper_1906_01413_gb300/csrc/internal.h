@@ -194,13 +194,18 @@ struct AdvDev {
     const double *Eb = nullptr;       // [n] background emissions
     double *Es64 = nullptr;           // [n] E / dz at the current control
     float *Es32 = nullptr;
-    // batch workspace (Pmax probes of the context precision; the same bytes hold Pws64 FP64 probes)
+    double *cf64 = nullptr;           // [2][5][ny][nx] column coefficients, tangent linear and adjoint (adv_coefs)
+    // batch workspace (Pmax probes of the context precision; the same bytes hold Pws64 FP64
+    // probes): the tracer fields, two of a mixed context's probes or three of FP64 ones
     int Pmax = 0, Pmax64 = 0, Pws64 = 0;
-    void *cA = nullptr, *cB = nullptr, *src = nullptr, *ebar = nullptr, *tmp = nullptr;
+    size_t fields_bytes = 0;
+    void *fields = nullptr, *src = nullptr, *ebar = nullptr, *tmp = nullptr;
     // FP64 outer-loop workspace
-    double *c64A = nullptr, *c64B = nullptr, *ebar64 = nullptr, *tmp64 = nullptr;   // tmp64: Pmax64 * n
+    double *c64A = nullptr, *c64B = nullptr, *c64X = nullptr, *ebar64 = nullptr, *tmp64 = nullptr;   // tmp64: Pmax64 * n
 };
 
+// Fills cf64 from the winds.
+cudaError_t adv_coefs(const AdvDev &m, cudaStream_t s);
 // Y = A W (+ W) for ncols columns (ld >= n), in FP64 or FP32 (per fp64); r
 // holds Pmax * p residuals of that type.
 cudaError_t adv_hvp(const AdvDev &m, bool fp64, const void *W, void *Y, int64_t ld, int ncols, int add_identity,
