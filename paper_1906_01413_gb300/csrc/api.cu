@@ -2196,10 +2196,13 @@ riot_status riot_sketchnet_create(riot_sketchnet **out, int32_t c_in, int32_t wi
         return true;
     };
     SketchWork &w = net->w;
+    w.group = sketchnet_group(m_out, r_max, batch_max);
+    const size_t ng = (size_t)w.group;
     if (!alloc(&net->params, np) || !alloc(&net->grad, np) || !alloc(&net->m1, np) || !alloc(&net->m2, np) ||
         !alloc(&w.Z, B * m * n) || !alloc(&w.gZ, B * m * n) || !alloc(&w.acts, (size_t)(depth - 1) * B * width * n) ||
-        !alloc(&w.g0, B * wide * n) || !alloc(&w.g1, B * wide * n) || !alloc(&w.R, n * m) || !alloc(&w.XE, n * m) ||
-        !alloc(&w.UtX, (size_t)r_max * m) || !alloc(&w.G, m * m) || !alloc(&w.E, m * m) || !alloc(&w.sc, 4 * B) ||
+        !alloc(&w.g0, B * wide * n) || !alloc(&w.g1, B * wide * n) || !alloc(&w.inner, ng * ((size_t)r_max + m) * m) ||
+        !alloc(&w.E, ng * m * m) || !alloc(&w.part, sketchnet_part_floats()) || !alloc(&w.sc, 4 * B) ||
+        !alloc(&w.gpart, sketchnet_gpart_doubles(net->net)) ||
         !alloc(&net->loss, 1)) {
         riot_sketchnet_destroy(net);
         return RIOT_ENOMEM;

@@ -241,9 +241,15 @@ struct SketchNet {
 };
 struct SketchWork {
     float *Z = nullptr, *acts = nullptr, *gZ = nullptr, *g0 = nullptr, *g1 = nullptr;
-    float *R = nullptr, *UtX = nullptr, *G = nullptr, *E = nullptr, *XE = nullptr;
-    double *sc = nullptr;   // 4 doubles per window
+    int group = 1;                          // windows whose loss is formed together (sketchnet_group)
+    float *inner = nullptr, *E = nullptr;   // per window of a group (r + m) x m inner products and m x m
+    float *part = nullptr;                  // their split sums (sketchnet_part_floats)
+    double *sc = nullptr;                   // 4 doubles per window
+    double *gpart = nullptr;                // partial weight gradients (sketchnet_gpart_doubles)
 };
+int sketchnet_group(int m, int r, int B);
+size_t sketchnet_part_floats();
+size_t sketchnet_gpart_doubles(const SketchNet &net);
 // Z (B x m x n) from x (B x c_in x n); hidden activations into acts ((depth-1) x B x width x n)
 cudaError_t sketchnet_forward(const SketchNet &net, const float *params, const float *x, int n, int B, float *Z,
                               bool bf16, float *acts, cudaStream_t s);
