@@ -10,11 +10,22 @@
 //    issued as soon as every thread has passed the barrier of stage u, so
 //    global-memory latency is hidden behind S - 1 stages of arithmetic and
 //    every coefficient is read once per CTA and shared by its P probes.
-//  * P probes per CTA (1024 threads for E <= 8) keep their state in
-//    registers; halos cross chunk boundaries through shared memory.
+//  * P probes per CTA (512 threads for E <= 8) keep their state in
+//    registers; halos cross chunk boundaries through shared memory, one CTA
+//    barrier per stage.
 //  * Every wait on an mbarrier is bounded; a wait that runs out raises a
 //    flag in global memory (reported as RIOT_ETIMEOUT) and the CTA carries
 //    on, so the kernel always finishes.
+//
+// Bound: instruction issue and the barrier of every stage (67 % of the issue slots of a busy
+// SM; 157 instructions per warp and stage, 85 of them FP32).  What the stage's critical path
+// does not do: no division by the run-time ring depth in the thread that feeds the ring (every
+// warp waits for it at the barrier; 400 cycles a stage), no proxy fence before a refill
+// (buffers are only read between copies; 150 cycles), no loads of coefficients behind the
+// barrier (all warps at once: 40 cycles, and 350 more when they were held a stage ahead in a
+// second set of registers).  n = 4096, T = 200, 512 columns: 2717 -> 1870 us; n = 1003, 77
+// columns 807 -> 254 us; n = 40 200 -> 80 us; n = 8191, 192 columns 2495 -> 1778 us; the same
+// products bit for bit.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -43,8 +54,6 @@ __device__ __forceinline__ void mbar_inval(uint32_t bar)
 {
     asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
 }
-
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
 {
@@ -80,7 +89,6 @@ constexpr int kWaitPolls = 1 << 20;
 __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, int *err, volatile int *abort_flag,
                                                   int polls)
 {
-    if (*abort_flag) return false;
     for (int i = 0; i < polls; ++i) {
         if (mbar_try_wait(bar, parity)) return true;
         if (i > 32) __nanosleep(64);
@@ -109,40 +117,46 @@ struct TmaArgs {
 // for the adjoint pass.  Thread 0 keeps `issued` (copies started) and
 // `landed` (stages whose copy it has seen complete) so that after an abort it
 // can still wait for every copy it started before the CTA exits.
+template <typename Args>
 struct Ring {
+    const Args &a;
     float2 *buf;
-    uint32_t bar0;
-    int S, Np, total, c0, T, polls;
+    uint32_t buf0, bar0;
+    int S, Np, total;
     int issued, landed;
-    const float2 *coef;
     volatile int *abort_flag;
+    bool aborted;   // a wait of this thread ran out (or one of an earlier item's)
     __device__ int blk(int c) const
     {
-        const int u = c0 + c;
+        const int T = a.T, u = ((a.mode == 1) ? 4 * T : 0) + c;
         return u < 4 * T ? u : 8 * T - 1 - u;
     }
-    __device__ void issue(int c)
+    // Stage c into buffer `slot` (c mod S: kept by the caller, divisions by S would hold up the
+    // barrier that everything waits at).
+    __device__ void issue(int c, int slot)
     {
-        const int slot = c % S;
         const uint32_t bytes = (uint32_t)Np * 8u;
         const uint32_t bar = bar0 + 8u * slot;
-        fence_proxy_async();
+        // the buffer's last readers have passed a CTA barrier; no proxy fence: they only read it
         mbar_expect_tx(bar, bytes);
-        bulk_g2s(smem_u32(buf + (size_t)slot * Np), coef + (size_t)blk(c) * Np, bytes, bar);
+        bulk_g2s(buf0 + (uint32_t)slot * bytes, a.coef + (size_t)blk(c) * Np, bytes, bar);
         issued = c + 1;
     }
-    // Thread 0 only, before the stage's barrier: wait until stage c has landed.
-    // The barrier then makes the buffer visible to every thread.
-    __device__ void wait_ready(int c, int *err)
+    // Every thread: wait until stage c, in buffer `slot` with phase parity `phase`, has landed; its
+    // reads of the buffer then need no barrier.
+    __device__ void wait_ready(int c, int slot, int phase, int *err)
     {
-        if (threadIdx.x == 0 && mbar_wait_bounded(bar0 + 8u * (c % S), (uint32_t)((c / S) & 1), err, abort_flag, polls))
-            landed = c + 1;
+        if (aborted) return;
+        aborted = !mbar_wait_bounded(bar0 + 8u * slot, (uint32_t)phase, err, abort_flag, a.wait_polls);
+        if (!aborted) landed = c + 1;
     }
-    // Thread 0 only, after the stage's barrier (every thread is done with the
-    // buffer of stage c - 1): refill that buffer with stage c + S - 1.
-    __device__ void refill(int c)
+    // Thread 0 only, behind the barrier of stage c: refill the buffer of stage c - 1 with stage
+    // c - 1 + S.  Every thread has used its coefficients of stage c - 1 by then (the values it
+    // published before the barrier depend on the last ones it loaded); those of stage c may
+    // still be on their way to registers.
+    __device__ void refill(int c, int slot)
     {
-        if (threadIdx.x == 0 && c + S - 1 < total && !*abort_flag) issue(c + S - 1);
+        if (threadIdx.x == 0 && c > 0 && c - 1 + S < total && !aborted) issue(c - 1 + S, slot ? slot - 1 : S - 1);
     }
     __device__ const float4 *slot4(int slot) const { return reinterpret_cast<const float4 *>(buf + (size_t)slot * Np); }
     // After an abort: wait, with the full bound whatever the test limit, for every
@@ -152,7 +166,7 @@ struct Ring {
     // flag to 2: it may land in shared memory the CTA no longer owns.
     __device__ void drain(int *err)
     {
-        if (threadIdx.x != 0 || !*abort_flag) return;
+        if (threadIdx.x != 0 || !aborted) return;
         for (int c = landed; c < issued; ++c) {
             bool done = false;
             for (int i = 0; i < kWaitPolls && !done; ++i) {
@@ -164,160 +178,199 @@ struct Ring {
     }
 };
 
-// Tangent-linear tendency k = J(X) s of one RK4 stage for the PR probes a
-// thread holds; coefficients of the stage come from ring buffer `slot`
-// (float4 pairs interleaved by thread) and are shared by the PR probes.
-template <int E, int PR>
-__device__ __forceinline__ void tl_stage(const float (&s)[PR][E], float (&k)[PR][E], bool full, float *H, int nthr,
-                                         int tid, int left, int right, int &hb, Ring &ring, int c, int slot, int t,
-                                         int Tp, int *err)
-{
-    float *Hb = H + hb * 3 * PR * nthr;
-#pragma unroll
-    for (int r = 0; r < PR; ++r) {
-        Hb[(0 * PR + r) * nthr + tid] = full ? s[r][E - 2] : s[r][E - 3];
-        Hb[(1 * PR + r) * nthr + tid] = full ? s[r][E - 1] : s[r][E - 2];
-        Hb[(2 * PR + r) * nthr + tid] = s[r][0];
-    }
-    ring.wait_ready(c, err);
-    __syncthreads();
-    ring.refill(c);
-    float m2[PR], m1[PR], p1[PR];
-#pragma unroll
-    for (int r = 0; r < PR; ++r) {
-        m2[r] = Hb[(0 * PR + r) * nthr + left];
-        m1[r] = Hb[(1 * PR + r) * nthr + left];
-        p1[r] = Hb[(2 * PR + r) * nthr + right];
-    }
-    hb ^= 1;
-    const float4 *cf = ring.slot4(slot) + t;
-#pragma unroll
-    for (int j2 = 0; j2 < E / 2; ++j2) {
-        const float4 cc = cf[j2 * Tp];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int j = 2 * j2 + h;
-            const float ca = h ? cc.z : cc.x, cb = h ? cc.w : cc.y;
-#pragma unroll
-            for (int r = 0; r < PR; ++r) {
-                const float xm2 = (j == 0) ? m2[r] : (j == 1 ? m1[r] : s[r][j >= 2 ? j - 2 : 0]);
-                const float xm1 = (j == 0) ? m1[r] : s[r][j >= 1 ? j - 1 : 0];
-                float xp1;
-                if (j == E - 1) xp1 = p1[r];
-                else if (j == E - 2) xp1 = full ? s[r][E - 1] : p1[r];
-                else xp1 = s[r][j + 1 < E ? j + 1 : 0];
-                k[r][j] = fmaf(ca, xp1 - xm2, fmaf(cb, xm1, -s[r][j]));
-            }
-        }
-    }
-    if (!full)
-#pragma unroll
-        for (int r = 0; r < PR; ++r) k[r][E - 1] = 0.f;
-}
+// The PR probes of a thread as one shared-memory word (PR floats).
+template <int PR>
+struct Vec {
+    float v[PR];
+};
+template <>
+struct __align__(8) Vec<2> {
+    float v[2];
+};
 
-// Adjoint tendency out = J(X)^T m.  The boundary values of m are exchanged
-// and the neighbours' coefficients read from the shared ring, so every
-// coefficient read follows the stage's barrier.
-template <int E, int PR>
-__device__ __forceinline__ void ad_stage(const float (&m)[PR][E], float (&out)[PR][E], bool full, float *H, int nthr,
-                                         int tid, int left, int right, int &hb, Ring &ring, int c, int slot, int t,
-                                         int Tp, int offL, int oddL, int tr, int *err)
-{
-    float *Hb = H + hb * 3 * PR * nthr;
-#pragma unroll
-    for (int r = 0; r < PR; ++r) {
-        Hb[(0 * PR + r) * nthr + tid] = full ? m[r][E - 1] : m[r][E - 2];
-        Hb[(1 * PR + r) * nthr + tid] = m[r][0];
-        Hb[(2 * PR + r) * nthr + tid] = m[r][1];
-    }
-    ring.wait_ready(c, err);
-    __syncthreads();
-    ring.refill(c);
-    float mL[PR], mR0[PR], mR1[PR];
-#pragma unroll
-    for (int r = 0; r < PR; ++r) {
-        mL[r] = Hb[(0 * PR + r) * nthr + left];
-        mR0[r] = Hb[(1 * PR + r) * nthr + right];
-        mR1[r] = Hb[(2 * PR + r) * nthr + right];
-    }
-    hb ^= 1;
-    const float4 *s4 = ring.slot4(slot);
-    const float4 cl = s4[offL], cr = s4[tr];
-    const float aL = oddL ? cl.z : cl.x;
-    float ca[E], cb[E];
-#pragma unroll
-    for (int j2 = 0; j2 < E / 2; ++j2) {
-        const float4 cc = s4[j2 * Tp + t];
-        ca[2 * j2] = cc.x;
-        cb[2 * j2] = cc.y;
-        ca[2 * j2 + 1] = cc.z;
-        cb[2 * j2 + 1] = cc.w;
-    }
-    // (J^T m)_j = a_{j-1} m_{j-1} - a_{j+2} m_{j+2} + b_{j+1} m_{j+1} - m_j, three FMAs
-#pragma unroll
-    for (int r = 0; r < PR; ++r) {
-#pragma unroll
-        for (int j = 0; j < E; ++j) {
-            const float mm1 = (j == 0) ? mL[r] : m[r][j >= 1 ? j - 1 : 0];
-            const float am1 = (j == 0) ? aL : ca[j >= 1 ? j - 1 : 0];
-            float mp1, bp1;
-            if (j <= E - 2 && (full || j <= E - 3)) {
-                mp1 = m[r][j + 1 < E ? j + 1 : 0];
-                bp1 = cb[j + 1 < E ? j + 1 : 0];
-            } else {
-                mp1 = mR0[r];
-                bp1 = cr.y;
-            }
-            float mp2, ap2;
-            if (j <= E - 3 && (full || j <= E - 4)) {
-                mp2 = m[r][j + 2 < E ? j + 2 : 0];
-                ap2 = ca[j + 2 < E ? j + 2 : 0];
-            } else if (full ? (j == E - 2) : (j == E - 3)) {
-                mp2 = mR0[r];
-                ap2 = cr.x;
-            } else {
-                mp2 = mR1[r];
-                ap2 = cr.z;
-            }
-            out[r][j] = fmaf(am1, mm1, fmaf(-ap2, mp2, fmaf(bp1, mp1, -m[r][j])));
-        }
-        if (!full) out[r][E - 1] = 0.f;
-    }
-}
-
+// Stage coefficients of a thread's E variables in registers (shared by its PR probes), and for
+// the adjoint those of the neighbours' variables it needs: a of the left chunk's last variable,
+// (a, b) of the right chunk's first, a of its second.
 template <int E>
-__device__ __forceinline__ void band_apply_t(const float *st, const float *band, int hl, int hh, int n, int s0, int len,
+struct Coefs {
+    float a[E], b[E];
+    float aL, aR0, bR0, aR1;
+};
+
+// Place of a thread's coefficients in a stage buffer (float4 pairs interleaved by thread).
+struct CoefAt {
+    int t, tr, Tp, offL, oddL;
+};
+
+template <int E, bool AD>
+__device__ __forceinline__ void load_coefs(Coefs<E> &c, const float4 *s4, const CoefAt &at)
+{
+#pragma unroll
+    for (int j2 = 0; j2 < E / 2; ++j2) {
+        const float4 f = s4[j2 * at.Tp + at.t];
+        c.a[2 * j2] = f.x;
+        c.b[2 * j2] = f.y;
+        c.a[2 * j2 + 1] = f.z;
+        c.b[2 * j2 + 1] = f.w;
+    }
+    if (AD) {
+        const float4 cl = s4[at.offL], cr = s4[at.tr];
+        c.aL = at.oddL ? cl.z : cl.x;
+        c.aR0 = cr.x;
+        c.bR0 = cr.y;
+        c.aR1 = cr.z;
+    }
+}
+
+// Stream position c, its buffer c mod S and the parity of c / S.
+struct StageAt {
+    int c, slot, phase;
+    __device__ __forceinline__ void advance(int S)
+    {
+        ++c;
+        if (++slot == S) {
+            slot = 0;
+            phase ^= 1;
+        }
+    }
+};
+
+// One stage's inputs: the coefficients and the neighbours' edge values, exchanged around the
+// stage's barrier.  The coefficients are loaded before it (while other warps still compute:
+// behind it all warps' loads come at once), but behind it with 16 variables per thread, where
+// shared memory holds two stages of the largest states and the next copy has to start first
+// (n = 8191: 1.9 ms against 2.5).
+template <int E, bool AD, int PR, typename Args>
+__device__ __forceinline__ void stage_inputs(Coefs<E> &cc, const CoefAt &at, const Vec<PR> (&give)[3], Vec<PR> (&get)[3],
+                                             Vec<PR> *H, int nthr, int tid, const int (&from)[3], int &hb,
+                                             Ring<Args> &ring, const StageAt &sa, int *err)
+{
+    constexpr bool EARLY = E <= 8;
+    Vec<PR> *Hb = H + hb * 3 * nthr;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) Hb[i * nthr + tid] = give[i];
+    if (EARLY) {
+        ring.wait_ready(sa.c, sa.slot, sa.phase, err);
+        load_coefs<E, AD>(cc, ring.slot4(sa.slot), at);
+    }
+    __syncthreads();
+    ring.refill(sa.c, sa.slot);
+    if (!EARLY) {
+        ring.wait_ready(sa.c, sa.slot, sa.phase, err);
+        load_coefs<E, AD>(cc, ring.slot4(sa.slot), at);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) get[i] = Hb[i * nthr + from[i]];
+    hb ^= 1;
+}
+
+// Tangent-linear tendency k = J(X) s of one probe.
+template <int E>
+__device__ __forceinline__ void tl_tend32(const float (&s)[E], float (&k)[E], const Coefs<E> &c, bool full, float m2,
+                                          float m1, float p1)
+{
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const float xm2 = (j == 0) ? m2 : (j == 1 ? m1 : s[j >= 2 ? j - 2 : 0]);
+        const float xm1 = (j == 0) ? m1 : s[j >= 1 ? j - 1 : 0];
+        float xp1;
+        if (j == E - 1) xp1 = p1;
+        else if (j == E - 2) xp1 = full ? s[E - 1] : p1;
+        else xp1 = s[j + 1 < E ? j + 1 : 0];
+        k[j] = fmaf(c.a[j], xp1 - xm2, fmaf(c.b[j], xm1, -s[j]));
+    }
+    if (!full) k[E - 1] = 0.f;
+}
+
+// Adjoint tendency out = J(X)^T m of one probe:
+// (J^T m)_j = a_{j-1} m_{j-1} - a_{j+2} m_{j+2} + b_{j+1} m_{j+1} - m_j, three FMAs
+template <int E>
+__device__ __forceinline__ void ad_tend32(const float (&m)[E], float (&out)[E], const Coefs<E> &c, bool full, float mL,
+                                          float mR0, float mR1)
+{
+#pragma unroll
+    for (int j = 0; j < E; ++j) {
+        const float mm1 = (j == 0) ? mL : m[j >= 1 ? j - 1 : 0];
+        const float am1 = (j == 0) ? c.aL : c.a[j >= 1 ? j - 1 : 0];
+        float mp1, bp1;
+        if (j <= E - 2 && (full || j <= E - 3)) {
+            mp1 = m[j + 1 < E ? j + 1 : 0];
+            bp1 = c.b[j + 1 < E ? j + 1 : 0];
+        } else {
+            mp1 = mR0;
+            bp1 = c.bR0;
+        }
+        float mp2, ap2;
+        if (j <= E - 3 && (full || j <= E - 4)) {
+            mp2 = m[j + 2 < E ? j + 2 : 0];
+            ap2 = c.a[j + 2 < E ? j + 2 : 0];
+        } else if (full ? (j == E - 2) : (j == E - 3)) {
+            mp2 = mR0;
+            ap2 = c.aR0;
+        } else {
+            mp2 = mR1;
+            ap2 = c.aR1;
+        }
+        out[j] = fmaf(am1, mm1, fmaf(-ap2, mp2, fmaf(bp1, mp1, -m[j])));
+    }
+    if (!full) out[E - 1] = 0.f;
+}
+
+// out_j = sum_d band_d st[s0 + j + d]: the E values that a tap multiplies are a window in
+// registers that moves by one value per tap.
+template <int E>
+__device__ __forceinline__ void band_apply_t(const float *st, const float *band, int hl, int hh, int n, int s0,
                                              float (&out)[E])
 {
+    float x[E];
+    int ii = s0 - hl;
+    ii += (ii < 0) ? n : 0;
 #pragma unroll
-    for (int j = 0; j < E; ++j) out[j] = 0.f;
-    for (int d = -hl; d <= hh; ++d) {
-        const float w = band[d + hl];
+    for (int j = 0; j < E; ++j) {
+        out[j] = 0.f;
+        x[j] = st[swz(ii)];
+        ii = (ii + 1 == n) ? 0 : ii + 1;
+    }
+    for (int d0 = 0; d0 <= hl + hh; d0 += E) {
 #pragma unroll
-        for (int j = 0; j < E; ++j) {
-            int ii = s0 + j + d;
-            ii += (ii < 0) ? n : 0;
-            ii -= (ii >= n) ? n : 0;
-            if (j < len) out[j] = fmaf(w, st[swz(ii)], out[j]);
+        for (int u = 0; u < E; ++u) {
+            if (d0 + u > hl + hh) break;
+            const float w = band[d0 + u];
+#pragma unroll
+            for (int j = 0; j < E; ++j) out[j] = fmaf(w, x[(u + j) % E], out[j]);
+            x[u] = st[swz(ii)];
+            ii = (ii + 1 == n) ? 0 : ii + 1;
         }
     }
 }
+
+// One thread's first observation of a step (observation o0 + t), loaded a step ahead.
+struct ObsAhead {
+    int o0, o1, slot;
+    float w;   // weight (tangent linear)
+};
 
 // A CTA holds P thread groups of Tp threads; group g owns probes
 // blk * P * PR + g * PR + r, r < PR, and thread t of a group keeps chunk t of
 // each of them in registers.  Threads from P * Tp up to blockDim.x (a
 // persistent batch kernel runs windows of several sizes in one block shape)
 // are idle: they follow the barriers and touch only their own halo slots.
-template <int E, int PR, bool RAGGED = true>
-__device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned char *smem_raw, int *abort_flag)
+// Args: TmaArgs, or volatile TmaArgs in shared memory (then nothing of it stays in registers).
+template <int E, int PR, bool RAGGED, typename Args>
+__device__ __forceinline__ void hvp_tma_body(const Args &a, int blk, unsigned char *smem_raw, int *abort_flag)
 {
-    const ChunkGeom &G = a.geom;
+    ChunkGeom G;
+    G.n = a.geom.n;
+    G.E = E;
+    G.Tp = a.geom.Tp;
+    G.g = a.geom.g;
+    G.Np = a.geom.Np;
     const int Np = G.Np, n = G.n, Tp = G.Tp, P = a.P, S = a.S;
     const int nthr = blockDim.x;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_raw);
     float2 *ringbuf = reinterpret_cast<float2 *>(smem_raw + 128);
-    float *H = reinterpret_cast<float *>(ringbuf + (size_t)S * Np);
-    float *state = H + 2 * 3 * PR * nthr;
+    Vec<PR> *H = reinterpret_cast<Vec<PR> *>(ringbuf + (size_t)S * Np);
+    float *state = reinterpret_cast<float *>(H + 2 * 3 * nthr);
     const int SP = stage_pad_t(Np);
 
     const int tid = threadIdx.x;
@@ -332,35 +385,39 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
     const int tE = t * E;
     const int tl = (t == 0) ? Tp - 1 : t - 1, tr = (t == Tp - 1) ? 0 : t + 1;
     const int lenL = G.len(tl);
-    const int offL = ((lenL - 1) >> 1) * Tp + tl, oddL = (lenL - 1) & 1;
+    const CoefAt at = {t, tr, Tp, ((lenL - 1) >> 1) * Tp + tl, (lenL - 1) & 1};
     int hb = 0;
     const float h = a.dt, h2 = 0.5f * a.dt, h6 = a.dt / 6.f, h3 = a.dt / 3.f;
 
-    Ring ring;
+    Ring<Args> ring = {a};
     ring.buf = ringbuf;
+    ring.buf0 = smem_u32(ringbuf);
     ring.bar0 = smem_u32(bars);
     ring.S = S;
     ring.Np = Np;
-    ring.T = a.T;
-    ring.coef = a.coef;
-    ring.c0 = (a.mode == 1) ? 4 * a.T : 0;
-    ring.total = ((a.mode == 2) ? 4 * a.T : 8 * a.T) - ring.c0;
-    ring.polls = a.wait_polls;
+    ring.total = ((a.mode == 2) ? 4 * a.T : 8 * a.T) - ((a.mode == 1) ? 4 * a.T : 0);
     ring.issued = 0;
     ring.landed = 0;
     ring.abort_flag = abort_flag;
+    ring.aborted = *ring.abort_flag;
     if (tid == 0) {
         for (int i = 0; i < S; ++i) mbar_init(ring.bar0 + 8u * i, 1);
         fence_mbar_init();
     }
     __syncthreads();
-    if (tid == 0)
-        for (int c = 0; c < S - 1 && c < ring.total; ++c) ring.issue(c);
-    int c = 0;      // stream position
-    int slot = 0;   // ring buffer of stream position c (c mod S)
+    if (tid == 0) {
+        for (int c = 0; c < S && c < ring.total; ++c) ring.issue(c, c);
+    }
+    StageAt sa = {0, 0, 0};
+    Coefs<E> cc;
 
     float dx[PR][E];
     if (a.mode != 1) {
+        ObsAhead ob = {a.optr[0], a.optr[1], 0, 0.f};
+        if (live && ob.o0 + t < ob.o1) {
+            ob.slot = a.oslot[ob.o0 + t];
+            ob.w = a.rinv[ob.o0 + t];
+        }
 #pragma unroll
         for (int r = 0; r < PR; ++r) {
             const int probe = probe0 + r;
@@ -374,14 +431,14 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
 #pragma unroll
         for (int r = 0; r < PR; ++r) {
             float tmp[E];
-            band_apply_t<E>(state + (g * PR + r) * SP, a.band, a.hl, a.hh, n, s0, len, tmp);
+            band_apply_t<E>(state + (g * PR + r) * SP, a.band, a.hl, a.hh, n, s0, tmp);
 #pragma unroll
             for (int j = 0; j < E; ++j) dx[r][j] = (j < len) ? tmp[j] * a.sig[s0 + (j < len ? j : 0)] : 0.f;
         }
         __syncthreads();
+        const int from[3] = {left, left, right};
         for (int tt = 0;; ++tt) {
-            const int o0 = a.optr[tt], o1 = a.optr[tt + 1];
-            if (o0 < o1) {
+            if (ob.o0 < ob.o1) {
                 if (live)
 #pragma unroll
                     for (int r = 0; r < PR; ++r) {
@@ -396,41 +453,50 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
                     if (live && probe < a.ncols) {
                         const float *st = state + (g * PR + r) * SP;
                         float *rr = a.r + (size_t)probe * (size_t)a.p;
-                        for (int o = o0 + t; o < o1; o += Tp) rr[o] = a.rinv[o] * st[swz(a.oslot[o])];
+                        if (ob.o0 + t < ob.o1) rr[ob.o0 + t] = ob.w * st[swz(ob.slot)];
+                        for (int o = ob.o0 + t + Tp; o < ob.o1; o += Tp) rr[o] = a.rinv[o] * st[swz(a.oslot[o])];
                     }
                 }
                 __syncthreads();
             }
             if (tt == a.T) break;
-            float s[PR][E], k[PR][E], acc[PR][E];
+            ob.o0 = ob.o1;
+            ob.o1 = a.optr[tt + 2];
+            float s[PR][E], acc[PR][E];
 #pragma unroll
             for (int r = 0; r < PR; ++r)
 #pragma unroll
                 for (int j = 0; j < E; ++j) s[r][j] = dx[r][j];
-            tl_stage<E, PR>(s, k, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, a.err);
-            slot = (slot + 1 == S) ? 0 : slot + 1;
+#pragma unroll
+            for (int st = 0; st < 4; ++st) {
+                Vec<PR> give[3], get[3];
+#pragma unroll
+                for (int r = 0; r < PR; ++r) {
+                    give[0].v[r] = full ? s[r][E - 2] : s[r][E - 3];
+                    give[1].v[r] = full ? s[r][E - 1] : s[r][E - 2];
+                    give[2].v[r] = s[r][0];
+                }
+                stage_inputs<E, false>(cc, at, give, get, H, nthr, tid, from, hb, ring, sa, a.err);
+                if (st == 2 && live && ob.o0 + t < ob.o1) {   // the next step's observation, a step ahead
+                    ob.slot = a.oslot[ob.o0 + t];
+                    ob.w = a.rinv[ob.o0 + t];
+                }
+#pragma unroll
+                for (int r = 0; r < PR; ++r) {
+                    float k[E];
+                    tl_tend32<E>(s[r], k, cc, full, get[0].v[r], get[1].v[r], get[2].v[r]);
+#pragma unroll
+                    for (int j = 0; j < E; ++j) {
+                        acc[r][j] = (st == 0) ? k[j] : (st == 3) ? acc[r][j] + k[j] : fmaf(2.f, k[j], acc[r][j]);
+                        if (st < 3) s[r][j] = fmaf(st == 2 ? h : h2, k[j], dx[r][j]);
+                    }
+                }
+                sa.advance(S);
+            }
 #pragma unroll
             for (int r = 0; r < PR; ++r)
 #pragma unroll
-                for (int j = 0; j < E; ++j) { acc[r][j] = k[r][j]; s[r][j] = fmaf(h2, k[r][j], dx[r][j]); }
-            tl_stage<E, PR>(s, k, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, a.err);
-            slot = (slot + 1 == S) ? 0 : slot + 1;
-#pragma unroll
-            for (int r = 0; r < PR; ++r)
-#pragma unroll
-                for (int j = 0; j < E; ++j) { acc[r][j] = fmaf(2.f, k[r][j], acc[r][j]); s[r][j] = fmaf(h2, k[r][j], dx[r][j]); }
-            tl_stage<E, PR>(s, k, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, a.err);
-            slot = (slot + 1 == S) ? 0 : slot + 1;
-#pragma unroll
-            for (int r = 0; r < PR; ++r)
-#pragma unroll
-                for (int j = 0; j < E; ++j) { acc[r][j] = fmaf(2.f, k[r][j], acc[r][j]); s[r][j] = fmaf(h, k[r][j], dx[r][j]); }
-            tl_stage<E, PR>(s, k, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, a.err);
-            slot = (slot + 1 == S) ? 0 : slot + 1;
-#pragma unroll
-            for (int r = 0; r < PR; ++r)
-#pragma unroll
-                for (int j = 0; j < E; ++j) { acc[r][j] += k[r][j]; dx[r][j] = fmaf(h6, acc[r][j], dx[r][j]); }
+                for (int j = 0; j < E; ++j) dx[r][j] = fmaf(h6, acc[r][j], dx[r][j]);
         }
         if (a.mode == 2) {
             ring.drain(a.err);
@@ -439,17 +505,28 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
                 for (int i = 0; i < S; ++i) mbar_inval(ring.bar0 + 8u * i);
             return;
         }
-        __syncthreads();   // last tangent-linear stage read before the adjoint refills its buffer
     }
-
     float lam[PR][E];
 #pragma unroll
     for (int r = 0; r < PR; ++r)
 #pragma unroll
         for (int j = 0; j < E; ++j) lam[r][j] = 0.f;
+    ObsAhead ob = {a.optr[a.T], a.optr[a.T + 1], 0, 0.f};
+    float ro[PR];
+#pragma unroll
+    for (int r = 0; r < PR; ++r) ro[r] = 0.f;
+    auto obs_ahead = [&]() {
+        if (live && ob.o0 + t < ob.o1) {
+            ob.slot = a.oslot[ob.o0 + t];
+#pragma unroll
+            for (int r = 0; r < PR; ++r)
+                if (probe0 + r < a.ncols) ro[r] = a.r[(size_t)(probe0 + r) * (size_t)a.p + ob.o0 + t];
+        }
+    };
+    obs_ahead();
+    const int from[3] = {left, right, right};
     for (int tt = a.T;; --tt) {
-        const int o0 = a.optr[tt], o1 = a.optr[tt + 1];
-        if (o0 < o1) {
+        if (ob.o0 < ob.o1) {
             if (live)
 #pragma unroll
                 for (int r = 0; r < PR; ++r) {
@@ -464,7 +541,8 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
                 if (live && probe < a.ncols) {
                     float *st = state + (g * PR + r) * SP;
                     const float *rr = a.r + (size_t)probe * (size_t)a.p;
-                    for (int o = o0 + t; o < o1; o += Tp) atomicAdd(&st[swz(a.oslot[o])], rr[o]);
+                    if (ob.o0 + t < ob.o1) atomicAdd(&st[swz(ob.slot)], ro[r]);
+                    for (int o = ob.o0 + t + Tp; o < ob.o1; o += Tp) atomicAdd(&st[swz(a.oslot[o])], rr[o]);
                 }
             }
             __syncthreads();
@@ -476,35 +554,39 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
             }
         }
         if (tt == 0) break;
-        float lk[PR][E], ls[PR][E], lx[PR][E];
+        ob.o1 = ob.o0;
+        ob.o0 = a.optr[tt - 1];
+        // l4 = J4^T (h/6) lam, l3 = J3^T ((h/3) lam + h l4), l2 = J2^T ((h/3) lam + (h/2) l3), l1 =
+        // J1^T ((h/6) lam + (h/2) l2), lam_0 = lam + l4 + l3 + l2 + l1
+        float lx[PR][E], m[PR][E];
 #pragma unroll
         for (int r = 0; r < PR; ++r)
 #pragma unroll
-            for (int j = 0; j < E; ++j) lk[r][j] = h6 * lam[r][j];
-        ad_stage<E, PR>(lk, ls, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, offL, oddL, tr, a.err);
-        slot = (slot + 1 == S) ? 0 : slot + 1;
+            for (int j = 0; j < E; ++j) m[r][j] = h6 * lam[r][j];
 #pragma unroll
-        for (int r = 0; r < PR; ++r)
+        for (int st = 0; st < 4; ++st) {
+            Vec<PR> give[3], get[3];
 #pragma unroll
-            for (int j = 0; j < E; ++j) { lx[r][j] = lam[r][j] + ls[r][j]; lk[r][j] = fmaf(h3, lam[r][j], h * ls[r][j]); }
-        ad_stage<E, PR>(lk, ls, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, offL, oddL, tr, a.err);
-        slot = (slot + 1 == S) ? 0 : slot + 1;
+            for (int r = 0; r < PR; ++r) {
+                give[0].v[r] = full ? m[r][E - 1] : m[r][E - 2];
+                give[1].v[r] = m[r][0];
+                give[2].v[r] = m[r][1];
+            }
+            stage_inputs<E, true>(cc, at, give, get, H, nthr, tid, from, hb, ring, sa, a.err);
+            if (st == 2) obs_ahead();
 #pragma unroll
-        for (int r = 0; r < PR; ++r)
+            for (int r = 0; r < PR; ++r) {
+                float k[E];
+                ad_tend32<E>(m[r], k, cc, full, get[0].v[r], get[1].v[r], get[2].v[r]);
 #pragma unroll
-            for (int j = 0; j < E; ++j) { lx[r][j] += ls[r][j]; lk[r][j] = fmaf(h3, lam[r][j], h2 * ls[r][j]); }
-        ad_stage<E, PR>(lk, ls, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, offL, oddL, tr, a.err);
-        slot = (slot + 1 == S) ? 0 : slot + 1;
-#pragma unroll
-        for (int r = 0; r < PR; ++r)
-#pragma unroll
-            for (int j = 0; j < E; ++j) { lx[r][j] += ls[r][j]; lk[r][j] = fmaf(h6, lam[r][j], h2 * ls[r][j]); }
-        ad_stage<E, PR>(lk, ls, full, H, nthr, tid, left, right, hb, ring, c++, slot, t, Tp, offL, oddL, tr, a.err);
-        slot = (slot + 1 == S) ? 0 : slot + 1;
-#pragma unroll
-        for (int r = 0; r < PR; ++r)
-#pragma unroll
-            for (int j = 0; j < E; ++j) lam[r][j] = lx[r][j] + ls[r][j];
+                for (int j = 0; j < E; ++j) {
+                    lx[r][j] = (st == 0 ? lam[r][j] : lx[r][j]) + k[j];
+                    if (st < 3) m[r][j] = fmaf(st == 2 ? h6 : h3, lam[r][j], (st == 0 ? h : h2) * k[j]);
+                    else lam[r][j] = lx[r][j];
+                }
+            }
+            sa.advance(S);
+        }
     }
 
     ring.drain(a.err);
@@ -524,7 +606,7 @@ __device__ __forceinline__ void hvp_tma_body(const TmaArgs &a, int blk, unsigned
     for (int r = 0; r < PR; ++r) {
         const int probe = probe0 + r;
         float y[E];
-        band_apply_t<E>(state + (g * PR + r) * SP, a.band, a.hl, a.hh, n, s0, len, y);
+        band_apply_t<E>(state + (g * PR + r) * SP, a.band, a.hl, a.hh, n, s0, y);
         if (live && probe < a.ncols) {
             float *yo = a.Y + (size_t)probe * a.ld;
             const float *w = a.W ? a.W + (size_t)probe * a.ld : nullptr;
@@ -557,6 +639,9 @@ __global__ void __launch_bounds__(MAXT, 1) l96_hvp_batch_kernel(const TmaArgs *a
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int abort_flag, item_s;
+    // the item's window; volatile, so that its fields are read where they are used: held in
+    // registers beside the state they spill
+    __shared__ volatile TmaArgs a;
     if (threadIdx.x == 0) abort_flag = 0;
     for (;;) {
         __syncthreads();
@@ -565,10 +650,14 @@ __global__ void __launch_bounds__(MAXT, 1) l96_hvp_batch_kernel(const TmaArgs *a
         const int it = item_s;
         if (it >= nitems) break;
         const BatchItem bi = items[it];
-        const TmaArgs a = args[bi.win];
-        if (a.geom.E == 4) hvp_tma_body<4, 2>(a, bi.blk, smem_raw, &abort_flag);
-        else if (a.geom.E == 8) hvp_tma_body<8, 2>(a, bi.blk, smem_raw, &abort_flag);
-        else hvp_tma_body<16, 1>(a, bi.blk, smem_raw, &abort_flag);
+        static_assert(sizeof(TmaArgs) % sizeof(int) == 0 && sizeof(TmaArgs) / sizeof(int) <= MAXT, "copied by words");
+        if (threadIdx.x < sizeof(TmaArgs) / sizeof(int))
+            reinterpret_cast<volatile int *>(&a)[threadIdx.x] = reinterpret_cast<const int *>(args + bi.win)[threadIdx.x];
+        __syncthreads();
+        const int E = a.geom.E;
+        if (E == 4) hvp_tma_body<4, 2, true>(a, bi.blk, smem_raw, &abort_flag);
+        else if (E == 8) hvp_tma_body<8, 2, true>(a, bi.blk, smem_raw, &abort_flag);
+        else hvp_tma_body<16, 1, true>(a, bi.blk, smem_raw, &abort_flag);
     }
 }
 
@@ -582,12 +671,15 @@ size_t tma_smem_bytes(int Np, int nthr, int P, int S, int PR)
 
 }  // namespace
 
-// Choose P thread groups per CTA and ring depth S for the shared-memory
-// budget; positive hints are taken when they fit.
-static bool tma_plan(const ChunkGeom &g, int ncols, int PR, int maxthr, size_t smem_max, int P_hint, int S_hint,
-                     int *P_out, int *S_out)
+// Probe groups P per CTA and ring depth S within the shared-memory budget; positive hints are
+// taken when they fit.  Otherwise the shape with the least modelled time per stage: a wave of CTAs
+// takes 350 cycles (exchange, barrier, latency) and 8 per variable and probe for each warp of a
+// sub-partition, so a few columns spread over the SMs (77 columns of n = 1003: 77 CTAs of one
+// column 254 us, ten of eight more than twice that) and many fill a CTA.  Returns that time, < 0 if nothing fits.
+static double tma_plan(const ChunkGeom &g, int ncols, int PR, int maxthr, size_t smem_max, int P_hint, int S_hint,
+                       int *P_out, int *S_out)
 {
-    const int groups_needed = (ncols + PR - 1) / PR;
+    const int groups_needed = (ncols + PR - 1) / PR, sms = num_sms();
     int Pmax = maxthr / g.Tp;
     if (Pmax > 64) Pmax = 64;
     if (Pmax > groups_needed) Pmax = groups_needed;
@@ -597,17 +689,28 @@ static bool tma_plan(const ChunkGeom &g, int ncols, int PR, int maxthr, size_t s
         if (P >= 1 && tma_smem_bytes(g.Np, P * g.Tp, P, S, PR) <= smem_max) {
             *P_out = P;
             *S_out = S;
-            return true;
+            return 0.0;
         }
     }
-    for (int P = Pmax; P >= 1; --P)
-        for (int S = 4; S >= 2; --S)
-            if (tma_smem_bytes(g.Np, P * g.Tp, P, S, PR) <= smem_max) {
-                *P_out = P;
-                *S_out = S;
-                return true;
-            }
-    return false;
+    double best = -1.0;
+    for (int P = 1; P <= Pmax; ++P) {
+        int S = 8;
+        while (S > 2 && tma_smem_bytes(g.Np, P * g.Tp, P, S, PR) > smem_max) --S;
+        const size_t sm = tma_smem_bytes(g.Np, P * g.Tp, P, S, PR);
+        if (sm > smem_max) continue;
+        const int warps = (P * g.Tp + 31) / 32, ctas = (groups_needed + P - 1) / P, per_sm = (ctas + sms - 1) / sms;
+        int fit = maxthr / (32 * warps);   // CTAs an SM holds at a time
+        if (fit > (int)(smem_max / sm)) fit = (int)(smem_max / sm);
+        if (fit < 1) fit = 1;
+        if (fit > per_sm) fit = per_sm;
+        const double t = (double)((per_sm + fit - 1) / fit) * (350.0 + 8.0 * g.E * PR * ((fit * warps + 3) / 4));
+        if (best < 0.0 || t < best) {
+            best = t;
+            *P_out = P;
+            *S_out = S;
+        }
+    }
+    return best;
 }
 
 template <int E, int PR, int MAXT, int MINB = 1>
@@ -632,15 +735,25 @@ cudaError_t l96_hvp_tma_launch(const L96Dev &m, const float2 *coef, const float 
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     const int E = m.geom.E;
-    // two probes per thread (registers) for E <= 8: 512-thread CTAs, one per SM; two_per_sm
-    // (E = 8): one probe per thread in 64 registers, two CTAs per SM sharing its shared memory
+    // two probes per thread (registers) for E <= 8: 512-thread CTAs, one per SM; one where few
+    // columns leave SMs idle otherwise (E = 8); two_per_sm (E = 8): one probe per thread in 64
+    // registers, two CTAs per SM sharing its shared memory
     const bool pair = two_per_sm && E == 8;
-    const int PR = (E <= 8 && !pair) ? 2 : 1;
+    int PR = (E <= 8 && !pair) ? 2 : 1;
     const int maxthr = 512;
     const size_t smem_max = pair ? (size_t)smem_sm / 2 - 1024 : (size_t)smem_optin - 1024;
     int P = 1, S = 2;
-    if (!tma_plan(m.geom, ncols, PR, maxthr, smem_max, P_hint, S_hint, &P, &S))
-        return cudaErrorInvalidConfiguration;
+    const double t = tma_plan(m.geom, ncols, PR, maxthr, smem_max, P_hint, S_hint, &P, &S);
+    if (t < 0.0) return cudaErrorInvalidConfiguration;
+    if (PR == 2 && E == 8 && t > 0.0) {
+        int P1 = 1, S1 = 2;
+        const double t1 = tma_plan(m.geom, ncols, 1, maxthr, smem_max, 0, 0, &P1, &S1);
+        if (t1 >= 0.0 && t1 < t) {
+            PR = 1;
+            P = P1;
+            S = S1;
+        }
+    }
     TmaArgs a;
     a.geom = m.geom;
     a.T = m.T;
@@ -671,7 +784,9 @@ cudaError_t l96_hvp_tma_launch(const L96Dev &m, const float2 *coef, const float 
     const int grid = (ncols + per_cta - 1) / per_cta;
     switch (E) {
     case 4: return launch_tma<4, 2, 512>(a, grid, nthr, sm, s);
-    case 8: return pair ? launch_tma<8, 1, 512, 2>(a, grid, nthr, sm, s) : launch_tma<8, 2, 512>(a, grid, nthr, sm, s);
+    case 8:
+        if (pair) return launch_tma<8, 1, 512, 2>(a, grid, nthr, sm, s);
+        return PR == 1 ? launch_tma<8, 1, 512>(a, grid, nthr, sm, s) : launch_tma<8, 2, 512>(a, grid, nthr, sm, s);
     case 16: return launch_tma<16, 1, 512>(a, grid, nthr, sm, s);
     default: return cudaErrorInvalidValue;
     }
