@@ -605,6 +605,7 @@ __device__ __forceinline__ void inviter_one(uint32_t i, const double *dd, const 
         }
     }
     u0[IDX(m - 1)] = rcp_fast((fabs(a_cur) < tiny) ? (a_cur < 0.0 ? -tiny : tiny) : a_cur);
+    u1[IDX(m - 1)] = u2[IDX(m - 1)] = 0.0;   // read by the substitution's first row, times zero
     // start vector: distinct pseudo-random values per eigenvalue
     for (int l = 0; l < m; ++l) z[l] = hash_uniform(i, (uint32_t)l) + 1e-3;
     for (int iter = 0; iter < 3; ++iter) {
@@ -751,6 +752,9 @@ __device__ __forceinline__ void inviter_warp(uint32_t i, const double *dd, const
             }
         }
         u0[m - 1] = rcp_fast(mag_ge(a_cur, tiny) ? a_cur : (a_cur < 0.0 ? -tiny : tiny));
+        // the substitution's first row multiplies these by zero: left unset, a NaN or infinity that
+        // another kernel had in this shared memory would spread to the whole vector
+        u1[m - 1] = u2[m - 1] = 0.0;
     }
     for (int l = lane; l < m; l += 32) z[l] = hash_uniform(i, (uint32_t)l) + 1e-3;
     __syncwarp();
