@@ -874,7 +874,7 @@ cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *
     unsigned char *piv = (unsigned char *)(work + 8 * kk);
     double *vec = work + 9 * kk;
     double *pq = vec, *d = vec + 4 * k, *e = vec + 5 * k;   // pq: p and q of two consecutive columns
-    double *e2 = vec + 6 * k, *w = vec + 7 * k, *tnorm = vec + 8 * k + 2;
+    double *e2 = vec + 6 * k, *w = vec + 7 * k, *tnorm = vec + 32 * k + 1008;   // in the gap before counts: no other piece within reach for k = 1, 2
     int *blo = (int *)(vec + 9 * k), *bhi = (int *)(vec + 10 * k);
     int *bstart = (int *)(vec + 11 * k), *nblocks = (int *)(vec + 12 * k);
     double *wrq = vec + 13 * k;
@@ -944,7 +944,7 @@ cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *
     // within about 1e-7, enough for vectors that are used in FP32 (fp32_vectors).
     // The Grams are split over K in the LU scratch of the inverse iteration.
     const int shifted = fp32_vectors ? 1 : 2;
-    if (fp32_vectors && tc_err) {
+    if (fp32_vectors && tc_err && k > 1) {   // k = 1: the Gram's scratch would reach into Zt32
         // vectors consumed in FP32: orthonormalise their FP32 rounding as the mixed path's
         // CholeskyQR does (exact tensor-core Gram, FP64 Cholesky, one-launch FP32 solve); the
         // LU scratch holds the FP32 copy and factor, the Gram's split integers, and pq the
