@@ -1124,7 +1124,7 @@ riot_status rsvd_eig(riot_ctx *ctx, int k)
     if (ctx->eig_method == RIOT_EIG_JACOBI)
         CU(jacobi_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->s));
     else
-        CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->s,
+        CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, ctx->s,
                        ctx->prec == RIOT_PREC_MIXED, ctx->prec == RIOT_PREC_MIXED ? ctx->errflag : nullptr));
     if (ctx->scale_exp) CU(scal(k, ldexp(1.0, ctx->scale_exp), ctx->lam, ctx->s));
     return RIOT_OK;
@@ -1292,8 +1292,8 @@ riot_status bfail(riot_batch *b, riot_status st, const char *fmt, ...)
 // Queue one inner loop (Algorithm 3: sketch, Y = A Omega, q power
 // iterations, Q, K, eigenpairs, Ritz vectors, increment) of every window of
 // the batch: per-window work on the window's branch stream, the Hessian
-// products of all windows in one persistent launch on the main stream, the
-// eigensolvers (cooperative, all SMs) one after another on the main stream.
+// products of all windows in one persistent launch on the main stream, and so
+// the tridiagonalisations (cooperative launches of as many windows as fit).
 riot_status batch_enqueue(riot_batch *b, int64_t sketch_stream)
 {
     const int nw = (int)b->ctx.size();
@@ -1339,18 +1339,35 @@ riot_status batch_enqueue(riot_batch *b, int64_t sketch_stream)
         }
         if (st != RIOT_OK || e != cudaSuccess) break;
         if (!fork()) break;
-        for (int w = 0; w < nw && st == RIOT_OK; ++w) st = rsvd_end(b->ctx[w], b->k[w], false);
-        if (st != RIOT_OK || !join()) break;
+        std::vector<TridiagJob> jobs;   // the windows' tridiagonalisations run side by side
+        for (int w = 0; w < nw && st == RIOT_OK && e == cudaSuccess; ++w) {
+            riot_ctx *c = b->ctx[w];
+            st = rsvd_end(c, b->k[w], false);
+            if (st == RIOT_OK && c->eig_method == RIOT_EIG_TRIDIAG) {
+                e = tridiag_prepare(c->Km, b->k[w], c->jwork, c->info + 12, c->s);
+                jobs.push_back({b->k[w], c->jwork, c->errflag});
+            }
+        }
+        if (st != RIOT_OK || e != cudaSuccess || !join()) break;
+        if ((e = tridiag_run(jobs.data(), (int)jobs.size(), b->main)) != cudaSuccess) break;
         for (int w = 0; w < nw && st == RIOT_OK; ++w) {
+            if (b->ctx[w]->eig_method == RIOT_EIG_TRIDIAG) continue;
             b->ctx[w]->s = b->main;
             st = rsvd_eig(b->ctx[w], b->k[w]);
             b->ctx[w]->s = b->ws[w];
         }
         if (st != RIOT_OK || !fork()) break;
-        for (int w = 0; w < nw && st == RIOT_OK; ++w) {
-            st = rsvd_ritz(b->ctx[w], b->k[w]);
-            if (st == RIOT_OK) st = increment_queue(b->ctx[w], b->k[w]);
+        for (int w = 0; w < nw && st == RIOT_OK && e == cudaSuccess; ++w) {
+            riot_ctx *c = b->ctx[w];
+            if (c->eig_method == RIOT_EIG_TRIDIAG) {
+                e = tridiag_finish(b->k[w], c->lam, c->Z, c->jwork, c->info + 12, c->s, true, c->errflag, false);
+                if (e == cudaSuccess && c->scale_exp) e = scal(b->k[w], ldexp(1.0, c->scale_exp), c->lam, c->s);
+                if (e != cudaSuccess) break;
+            }
+            st = rsvd_ritz(c, b->k[w]);
+            if (st == RIOT_OK) st = increment_queue(c, b->k[w]);
         }
+        if (e != cudaSuccess) break;
         if (st != RIOT_OK) break;
         join();
     } while (0);
@@ -1914,14 +1931,16 @@ riot_status riot_symm_eig(const double *K_dev, int32_t k, double *lambda_dev, do
     }
     riot_status st = RIOT_OK;
     cudaError_t e = cudaMemcpyAsync(Kc, K_dev, (size_t)k * k * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(info, 0, 4 * sizeof(int), s);
     if (e == cudaSuccess)
         e = (method == RIOT_EIG_JACOBI) ? jacobi_eig(Kc, k, lambda_dev, Z_dev, work, info, s)
-                                        : tridiag_eig(Kc, k, lambda_dev, Z_dev, work, info, s);
-    int h[2] = {0, 0};
+                                        : tridiag_eig(Kc, k, lambda_dev, Z_dev, work, info, info + 2, s);
+    int h[3] = {0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) st = RIOT_ECUDA;
     else if (method == RIOT_EIG_JACOBI && h[0] < 0) st = RIOT_ENOCONV;
+    else if (method == RIOT_EIG_TRIDIAG && h[2]) st = RIOT_ETIMEOUT;
     else if (method == RIOT_EIG_TRIDIAG && (h[0] || h[1])) st = RIOT_ENOCONV;
     cudaFree(work);
     cudaFree(Kc);
@@ -2463,7 +2482,7 @@ static riot_status varcg_body(riot_ctx *ctx, int32_t m, double *dv_dev, double *
     // T_m, its eigenpairs (theta, Z), U = Q Z, dv = -U diag(1 / (1 + theta)) U^T g
     CU(cudaMemcpyAsync(betas_dev, betas.data(), sizeof(double) * mm, cudaMemcpyHostToDevice, s));
     CU(tridiag_fill(mm, alphas, betas_dev, ctx->Km, s));
-    CU(tridiag_eig(ctx->Km, mm, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, s));
+    CU(tridiag_eig(ctx->Km, mm, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s));
     int einfo[2] = {0, 0};
     CU(cudaMemcpyAsync(einfo, ctx->info + 12, sizeof(einfo), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
@@ -2491,7 +2510,7 @@ static riot_status varcg_body(riot_ctx *ctx, int32_t m, double *dv_dev, double *
 static riot_status small_eig(riot_ctx *ctx, int k, const char *what)
 {
     cudaStream_t s = ctx->s;
-    CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, s));
+    CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s));
     int einfo[2] = {0, 0};
     CU(cudaMemcpyAsync(einfo, ctx->info + 12, sizeof(einfo), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));

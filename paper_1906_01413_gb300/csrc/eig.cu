@@ -3,8 +3,8 @@
 // every stage spreads its work over all SMs and the number of grid-wide
 // synchronisations is O(k), not O(k x sweeps).
 //
-//  1. Householder tridiagonalisation Q^T K Q = T in one cooperative launch,
-//     one grid barrier per column: every CTA derives the next reflector
+//  1. Householder tridiagonalisation Q^T K Q = T in one cooperative launch
+//     (of several problems side by side), one barrier per column: every CTA derives the next reflector
 //     itself, and each warp's rank-2 update of a column is followed at once
 //     by that column's product with the next reflector; Q is accumulated as
 //     Q^T on the fly.
@@ -21,6 +21,9 @@
 #include <float.h>
 #include <math.h>
 #include <stdint.h>
+
+#include <algorithm>
+#include <vector>
 
 #include "fp64_rcp.cuh"
 #include "internal.h"
@@ -121,6 +124,7 @@ __device__ void block_house(const double *col, int k, int r0, double *vs, double
 // the next column's p or q.  Column j + 1 itself is left to the CTAs (each
 // derives it), so no CTA writes what another still reads.  p and q are
 // double-buffered across the barrier.
+// b, G: this CTA's number and the CTAs of the problem; sync: a barrier over them.
 // RES (k <= 4 x CTAs): warp w < 4 of CTA b owns column b + G w of A and warp
 // 4 + w column b + G w of Q^T (G CTAs) for the whole run, kept in shared memory,
 // so each sub-partition carries at most one A column (a rank-2 update, two FMAs
@@ -129,19 +133,19 @@ __device__ void block_house(const double *col, int k, int r0, double *vs, double
 // published one step ahead), the last 2 x 2 block and Q^T at the end go back to
 // global memory.  Otherwise warps stride over the columns in global memory (L2),
 // four loads in flight per lane.
-template <bool RES>
-__global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int k, double *pq, double *d, double *e)
+template <bool RES, typename Sync>
+__device__ __forceinline__ void tridiag_body(double *A, double *Qt, int k, double *pq, double *d, double *e, int b, int G,
+                                             Sync sync)
 {
-    cg::grid_group grid = cg::this_grid();
     extern __shared__ double sm[];
     double *vcur = sm, *vnext = sm + k, *w = sm + 2 * k, *colj = sm + 3 * k, *red = sm + 4 * k;
     double *own = sm + 4 * k + kRedDoubles + (size_t)(threadIdx.x >> 5) * k;   // RES: this warp's column
     __shared__ double bcur_s, bnext_s, enext_s;
     const int lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int nw = gridDim.x * (blockDim.x >> 5);
+    const int gw = b * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const int nw = G * (blockDim.x >> 5);
     if (k < 3) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (b == 0 && threadIdx.x == 0) {
             d[0] = A[0];
             if (k == 2) {
                 e[0] = A[1];
@@ -152,7 +156,7 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
     }
     // RES: owned column (A column ocol for warps 0-3, Q^T column ocol for warps 4-7) into
     // shared memory
-    const int wib = threadIdx.x >> 5, ocol = blockIdx.x + gridDim.x * (wib & 3);
+    const int wib = threadIdx.x >> 5, ocol = b + G * (wib & 3);
     const bool ownA = RES && wib < 4 && ocol < k, ownQ = RES && wib >= 4 && ocol < k;
     if (RES && (ownA || ownQ)) {
         const double *src = ownA ? A + (int64_t)ocol * k : Qt + (int64_t)ocol * k;
@@ -161,7 +165,7 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
     }
     // reflector 0 from column 0, and its p, q
     block_house(A, k, 1, vcur, &bcur_s, &enext_s, red);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (b == 0 && threadIdx.x == 0) {
         d[0] = A[0];
         e[0] = enext_s;
     }
@@ -179,7 +183,7 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
             }
         }
     }
-    grid.sync();
+    sync();
     for (int j = 0; j + 2 < k; ++j) {
         const int r0 = j + 1, m = k - r0, par = j & 1;
         const bool next = (j + 3 < k);   // another reflector follows (column j + 1 has rows below r0 + 1)
@@ -212,7 +216,7 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
             block_house(colj, k, r0 + 1, vnext, &bnext_s, &enext_s, red, RES);
             __syncthreads();
             if constexpr (!RES) bn = bnext_s;
-            if (blockIdx.x == 0 && threadIdx.x == 0) {
+            if (b == 0 && threadIdx.x == 0) {
                 d[r0] = colj[r0];
                 e[r0] = enext_s;
             }
@@ -322,7 +326,7 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
         }
         for (int l = threadIdx.x; l < k; l += blockDim.x) vcur[l] = vnext[l];
         if (threadIdx.x == 0) bcur_s = bn;
-        grid.sync();
+        sync();
     }
     if constexpr (RES) {
         if (ownQ) {
@@ -330,12 +334,65 @@ __global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int
             for (int l = lane; l < k; l += 32) dst[l] = own[l];
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (b == 0 && threadIdx.x == 0) {
         // last 2 x 2 block
         d[k - 2] = A[(k - 2) + (int64_t)(k - 2) * k];
         e[k - 2] = A[(k - 1) + (int64_t)(k - 2) * k];
         d[k - 1] = A[(k - 1) + (int64_t)(k - 1) * k];
     }
+}
+
+__global__ void __launch_bounds__(256) tridiag_kernel(double *A, double *Qt, int k, double *pq, double *d, double *e)
+{
+    cg::grid_group grid = cg::this_grid();
+    tridiag_body<false>(A, Qt, k, pq, d, e, blockIdx.x, gridDim.x, [&]() { grid.sync(); });
+}
+
+// Several problems in one cooperative launch (all CTAs resident): problem p has the CTAs cta0 ..
+// cta0 + G - 1, a quarter of its columns each, and a barrier of its own, a counter that its CTAs
+// count up.  A column costs a problem 5 to 6 us, most of it the latency of two block sums, the
+// reflector's scalars and the barrier, so problems side by side take the time of the largest:
+// 48 batched windows (k up to 512) took 104 ms with their eigensolvers one after another and take
+// 61 so (the rest of each eigensolver on its window's stream).  The arithmetic of a problem does
+// not depend on G.
+struct TridiagProb {
+    double *A, *Qt, *pq, *d, *e;
+    unsigned *bar;   // zero at launch
+    int *err;        // raised if a wait at the barrier ran out
+    int k, cta0, G;
+};
+constexpr int kTridiagProbs = 48;
+struct TridiagProbs {
+    TridiagProb p[kTridiagProbs];
+    int n;
+};
+constexpr int kBarrierPolls = 1 << 20;   // about half a second
+
+__global__ void __launch_bounds__(256) tridiag_group_kernel(const __grid_constant__ TridiagProbs a)
+{
+    int i = 0;
+    while (i + 1 < a.n && (int)blockIdx.x >= a.p[i + 1].cta0) ++i;
+    const TridiagProb &p = a.p[i];
+    unsigned target = 0;   // thread 0's
+    bool dead = false;
+    auto sync = [&]() {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            target += (unsigned)p.G;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
+            unsigned seen = 0;
+            for (int t = 0; !dead; ++t) {
+                asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(p.bar) : "memory");
+                if (seen >= target) break;
+                if (t == kBarrierPolls) {
+                    dead = true;   // later waits return at once; the result is wrong and flagged
+                    atomicMax(p.err, 1);
+                }
+            }
+        }
+        __syncthreads();
+    };
+    tridiag_body<true>(p.A, p.Qt, p.k, p.pq, p.d, p.e, blockIdx.x - p.cta0, p.G, sync);
 }
 
 // Split T where |e_l| <= eps (|d_l| + |d_{l+1}|); block bounds per index; e^2;
@@ -865,44 +922,143 @@ __global__ void eig_sort_kernel(const double *w, const double *Zt, int k, double
 
 }  // namespace
 
-cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, cudaStream_t s,
-                        bool fp32_vectors, int *tc_err)
+namespace {
+
+// Places of one eigenproblem's pieces in its workspace (eig_work_doubles).
+struct EigWork {
+    double *A, *Qt, *Zt, *Zs, *u0, *u1, *u2, *ml, *vec, *pq, *d, *e, *e2, *w, *tnorm, *wrq, *ds, *e2s, *tsc, *dinv;
+    unsigned char *piv;
+    int *blo, *bhi, *bstart, *nblocks, *counts;
+    unsigned *bar;
+    EigWork(double *work, int k)
+    {
+        const size_t kk = (size_t)k * k;
+        A = work;
+        Qt = work + kk;
+        Zt = work + 2 * kk;
+        Zs = work + 3 * kk;
+        u0 = work + 4 * kk;
+        u1 = work + 5 * kk;
+        u2 = work + 6 * kk;
+        ml = work + 7 * kk;
+        piv = (unsigned char *)(work + 8 * kk);
+        vec = work + 9 * kk;
+        pq = vec;   // p and q of two consecutive columns
+        d = vec + 4 * k;
+        e = vec + 5 * k;
+        e2 = vec + 6 * k;
+        w = vec + 7 * k;
+        tnorm = vec + 32 * k + 1008;   // with bar in the gap before counts: no other piece within reach for k = 1, 2
+        blo = (int *)(vec + 9 * k);
+        bhi = (int *)(vec + 10 * k);
+        bstart = (int *)(vec + 11 * k);
+        nblocks = (int *)(vec + 12 * k);
+        wrq = vec + 13 * k;
+        ds = vec + 14 * k;   // scaled copies for the Sturm counts
+        e2s = vec + 15 * k;
+        tsc = vec + 16 * k;
+        bar = (unsigned *)(vec + 32 * k + 1016);   // the barrier's counter, in the gap before counts
+        counts = (int *)(vec + 32 * k + 1024);
+        dinv = vec + 32 * k + 1024 + ((size_t)kGrid * k + 1) / 2 + 8;
+    }
+};
+
+size_t tridiag_smem(int k, bool res)
 {
-    const size_t kk = (size_t)k * k;
-    double *A = work, *Qt = work + kk, *Zt = work + 2 * kk, *Zs = work + 3 * kk;
-    double *u0 = work + 4 * kk, *u1 = work + 5 * kk, *u2 = work + 6 * kk, *ml = work + 7 * kk;
-    unsigned char *piv = (unsigned char *)(work + 8 * kk);
-    double *vec = work + 9 * kk;
-    double *pq = vec, *d = vec + 4 * k, *e = vec + 5 * k;   // pq: p and q of two consecutive columns
-    double *e2 = vec + 6 * k, *w = vec + 7 * k, *tnorm = vec + 32 * k + 1008;   // in the gap before counts: no other piece within reach for k = 1, 2
-    int *blo = (int *)(vec + 9 * k), *bhi = (int *)(vec + 10 * k);
-    int *bstart = (int *)(vec + 11 * k), *nblocks = (int *)(vec + 12 * k);
-    double *wrq = vec + 13 * k;
-    double *ds = vec + 14 * k, *e2s = vec + 15 * k, *tsc = vec + 16 * k;   // scaled copies for the Sturm counts
-    int *counts = (int *)(vec + 32 * k + 1024);
-    double *dinv = vec + 32 * k + 1024 + ((size_t)kGrid * k + 1) / 2 + 8;
+    return sizeof(double) * (4 * (size_t)k + kRedDoubles + (res ? 8 * (size_t)k : 0));
+}
+
+}  // namespace
+
+// columns resident in shared memory when every column has a warp of its own on one CTA per SM
+bool tridiag_resident(int k) { return 2 * k <= num_sms() * 8; }
+
+cudaError_t tridiag_prepare(const double *K, int k, double *work, int *info, cudaStream_t s)
+{
+    const EigWork w(work, k);
     cudaError_t err;
     if ((err = cudaMemsetAsync(info, 0, 2 * sizeof(int), s)) != cudaSuccess) return err;
-    if ((err = cudaMemsetAsync(vec, 0, sizeof(double) * 9 * k, s)) != cudaSuccess) return err;
+    if ((err = cudaMemsetAsync(w.vec, 0, sizeof(double) * 9 * k, s)) != cudaSuccess) return err;
+    if ((err = cudaMemsetAsync(w.bar, 0, sizeof(unsigned), s)) != cudaSuccess) return err;
     count_launch();
-    eig_init_kernel<<<256, 256, 0, s>>>(K, k, A, Qt);
-    if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    {
-        const int grid = num_sms();   // one CTA per SM keeps the grid barrier short
-        // columns resident in shared memory when every column has a warp of its own
-        const bool res = 2 * k <= grid * 8;
-        const size_t smem = sizeof(double) * (4 * (size_t)k + kRedDoubles + (res ? 8 * (size_t)k : 0));
-        const void *fn = res ? (const void *)tridiag_kernel<true> : (const void *)tridiag_kernel<false>;
-        if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    eig_init_kernel<<<256, 256, 0, s>>>(K, k, w.A, w.Qt);
+    return cudaGetLastError();
+}
+
+cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
+{
+    cudaError_t err;
+    const int sms = num_sms();
+    std::vector<TridiagJob> order;
+    for (int i = 0; i < njobs; ++i) {
+        if (tridiag_resident(jobs[i].k)) {
+            order.push_back(jobs[i]);
+            continue;
+        }
+        // large problems: one at a time over all SMs, columns in global memory
+        EigWork w(jobs[i].work, jobs[i].k);
+        int k = jobs[i].k, per_sm = 0;
+        const size_t smem = tridiag_smem(k, false);
+        const void *fn = (const void *)tridiag_kernel;
+        if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+            (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
             return err;
-        int per_sm = 0;
-        if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess) return err;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
-        void *args[] = {&A, &Qt, &k, &pq, &d, &e};
+        void *args[] = {&w.A, &w.Qt, &k, &w.pq, &w.d, &w.e};
         count_launch();
-        err = cudaLaunchCooperativeKernel(fn, grid, 256, args, smem, s);
-        if (err != cudaSuccess) return err;
+        if ((err = cudaLaunchCooperativeKernel(fn, sms, 256, args, smem, s)) != cudaSuccess) return err;
     }
+    // the others by decreasing size, as many side by side as two CTAs per SM hold
+    std::stable_sort(order.begin(), order.end(), [](const TridiagJob &x, const TridiagJob &y) { return x.k > y.k; });
+    for (size_t at = 0; at < order.size();) {
+        TridiagProbs a;
+        a.n = 0;
+        const size_t smem = tridiag_smem(order[at].k, true);
+        const void *fn = (const void *)tridiag_group_kernel;
+        int per_sm = 0, ctas = 0;
+        if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+            (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
+            return err;
+        if (per_sm < 1) return cudaErrorInvalidConfiguration;
+        const int room = sms * (per_sm < 2 ? per_sm : 2);
+        while (at < order.size() && a.n < kTridiagProbs) {
+            const TridiagJob &j = order[at];
+            const int G = (j.k + 3) / 4;
+            if (a.n > 0 && ctas + G > room) break;
+            const EigWork w(j.work, j.k);
+            a.p[a.n++] = {w.A, w.Qt, w.pq, w.d, w.e, w.bar, j.err, j.k, ctas, G};
+            ctas += G;
+            ++at;
+        }
+        // alone, a problem takes every SM: fewer columns per CTA (k = 512: 3.32 ms, 3.43 on 128)
+        if (a.n == 1 && ctas < sms) a.p[0].G = ctas = sms;
+        void *args[] = {&a};
+        count_launch();
+        if ((err = cudaLaunchCooperativeKernel(fn, ctas, 256, args, smem, s)) != cudaSuccess) return err;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, int *err, cudaStream_t s,
+                        bool fp32_vectors, int *tc_err)
+{
+    cudaError_t e = tridiag_prepare(K, k, work, info, s);
+    const TridiagJob job = {k, work, err};
+    if (e == cudaSuccess) e = tridiag_run(&job, 1, s);
+    return e == cudaSuccess ? tridiag_finish(k, lam, Z, work, info, s, fp32_vectors, tc_err, true) : e;
+}
+
+cudaError_t tridiag_finish(int k, double *lam, double *Z, double *work, int *info, cudaStream_t s, bool fp32_vectors,
+                           int *tc_err, bool whole_gpu)
+{
+    const size_t kk = (size_t)k * k;
+    const EigWork ew(work, k);
+    double *Qt = ew.Qt, *Zt = ew.Zt, *Zs = ew.Zs, *u0 = ew.u0, *u1 = ew.u1, *u2 = ew.u2, *ml = ew.ml, *pq = ew.pq,
+           *d = ew.d, *e = ew.e, *e2 = ew.e2, *w = ew.w, *tnorm = ew.tnorm, *wrq = ew.wrq, *ds = ew.ds, *e2s = ew.e2s,
+           *tsc = ew.tsc, *dinv = ew.dinv;
+    unsigned char *piv = ew.piv;
+    int *blo = ew.blo, *bhi = ew.bhi, *bstart = ew.bstart, *nblocks = ew.nblocks, *counts = ew.counts;
+    cudaError_t err;
     count_launch();
     split_kernel<<<1, 1024, 0, s>>>(d, e, k, e2, blo, bhi, tnorm, bstart, nblocks, ds, e2s, tsc);
     count_launch();
@@ -958,7 +1114,7 @@ cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *
                                      : 0.0;
             if ((err = tc_gram_f32(k, k, Zt32, k, Zs, k, u0, tc_err, s)) != cudaSuccess) return err;
             if ((err = equilibrate(Zs, k, k, Zt32, 'f', k, k, pq, s)) != cudaSuccess) return err;
-            if ((err = cholesky(Zs, k, k, shift, info + (pass < shifted ? 0 : 1), dinv, s)) != cudaSuccess) return err;
+            if ((err = cholesky(Zs, k, k, shift, info + (pass < shifted ? 0 : 1), dinv, s, whole_gpu)) != cudaSuccess) return err;
             if ((err = convert_block(Zs, 'd', k, L32, 'f', k, k, k, s)) != cudaSuccess) return err;
             if ((err = put_block_inverses(L32, k, k, dinv, s)) != cudaSuccess) return err;
             if ((err = strsm_right_lt_inv(Zt32, k, k, k, L32, k, s)) != cudaSuccess) return err;
@@ -969,7 +1125,7 @@ cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *
             const double shift =
                 pass < shifted ? 11.0 * ((double)k * k + (double)k * (k + 1)) * ldexp(1.0, -53) : 0.0;
             if ((err = gram_lower(k, k, Zt, 'd', k, Zs, k, s, u0, 4 * kk)) != cudaSuccess) return err;
-            if ((err = cholesky(Zs, k, k, shift, info + (pass < shifted ? 0 : 1), dinv, s)) != cudaSuccess)
+            if ((err = cholesky(Zs, k, k, shift, info + (pass < shifted ? 0 : 1), dinv, s, whole_gpu)) != cudaSuccess)
                 return err;
             if ((err = trsm_right_lt(Zt, k, k, k, Zs, k, s, dinv)) != cudaSuccess) return err;
         }

@@ -345,8 +345,21 @@ size_t jacobi_work_doubles(int k);
 // stops at about 1e-7 (one shifted CholeskyQR pass less); with tc_err (the flag of the
 // tensor-core kernels' bounded waits) it runs on their FP32 rounding with the exact
 // tensor-core Gram and the one-launch FP32 solve, as the mixed path's CholeskyQR does
-cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, cudaStream_t s,
+// err: raised if a wait at the tridiagonalisation's barrier ran out.
+cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, int *err, cudaStream_t s,
                         bool fp32_vectors = false, int *tc_err = nullptr);
+// The same in three parts, so that several problems tridiagonalise side by side in one
+// cooperative launch: prepare, run and finish on each problem's workspace; prepare and finish may
+// be on parallel streams (whole_gpu false then, as for cholesky).
+struct TridiagJob {
+    int k;
+    double *work;
+    int *err;
+};
+cudaError_t tridiag_prepare(const double *K, int k, double *work, int *info, cudaStream_t s);
+cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s);
+cudaError_t tridiag_finish(int k, double *lam, double *Z, double *work, int *info, cudaStream_t s, bool fp32_vectors,
+                           int *tc_err, bool whole_gpu);
 size_t eig_work_doubles(int k);
 // elementwise helpers
 cudaError_t symmetrize(double *A, int k, int64_t lda, cudaStream_t s);
