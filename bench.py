@@ -406,13 +406,13 @@ def bench_bc_transport(R, torch, dev, flush, hbm_peak, ncols=128, reps=2):
     ncells = cfg.nx * cfg.ny * cfg.nz
     bytes_per_hvp = 8.0 * ncells * cfg.T * 2
     # measured DRAM bytes of one step of one column, times the 2T steps of a product
-    step_bytes, bc_note = profiled_traffic("adv_step_f2_kernel_bc_192x192x30_P32.md", "advdiff.cu")
+    step_bytes, bc_note = profiled_traffic("adv_step_z_kernel_bc_192x192x30_P32.md", "advdiff.cu")
     bc_traffic = None if step_bytes is None else step_bytes * 2 * cfg.T
     achieved = bytes_per_hvp * ncols / (ms * 1e-3) / 1e9
     return {"workload": "bc_%dx%dx%d_T%d_obs%d_blocks%d" % (cfg.nx, cfg.ny, cfg.nz, cfg.T, p, cfg.nblocks),
             "value": ncols / (ms * 1e-3), "unit": "HVP/s", "ms_per_hvp": ms / ncols, "columns_per_call": ncols,
             "dtype": "f32",
-            "roofline": {"bound": "hbm", "kernel": "adv_step_f2_kernel<15,32,8> (whole product timed)",
+            "roofline": {"bound": "hbm", "kernel": "adv_step_z_kernel<12,3> (whole product timed)",
                          "achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,
                          "traffic": bc_traffic, "traffic_source": bc_note, "bytes_per_hvp": bytes_per_hvp,
                          "bytes_basis": "one FP32 read and write of the tracer per RK4 step, TL and AD"}}
@@ -422,7 +422,7 @@ def bench_bc_inner_loop(R, torch, dev, flush):
     """One RIOT inner loop of the tracer inversion on its full grid (Algorithm 3 with k = 1024,
     q = 1: 2048 Hessian-vector products, CholeskyQR, K, the 1024 x 1024 FP64 eigensolver, Ritz
     vectors, increment), mixed precision, timed once with CUDA events after an L2 flush (one
-    inner loop is about 2048 x 6.7 ms of products)."""
+    inner loop is about 2048 x 2.7 ms of products)."""
     cfg = bc_synth.bc_large()
     ctx, xb, p = build_bc_problem(R, torch, cfg, dev, R.RIOT_PREC_MIXED, cfg.k)
     R.riot_outer_begin(ctx.h, xb)
