@@ -399,12 +399,14 @@ __device__ __forceinline__ void hvp_tma_body(const Args &a, int blk, unsigned ch
     ring.issued = 0;
     ring.landed = 0;
     ring.abort_flag = abort_flag;
-    ring.aborted = *ring.abort_flag;
     if (tid == 0) {
         for (int i = 0; i < S; ++i) mbar_init(ring.bar0 + 8u * i, 1);
         fence_mbar_init();
     }
     __syncthreads();
+    // behind the barrier: the flag is thread 0's store, and what the shared word held before it
+    // (whatever an earlier kernel left) would end every wait of this thread at once
+    ring.aborted = *ring.abort_flag;
     if (tid == 0) {
         for (int c = 0; c < S && c < ring.total; ++c) ring.issue(c, c);
     }
