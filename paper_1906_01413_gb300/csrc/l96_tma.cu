@@ -137,7 +137,8 @@ struct Ring {
     {
         const uint32_t bytes = (uint32_t)Np * 8u;
         const uint32_t bar = bar0 + 8u * slot;
-        // the buffer's last readers have passed a CTA barrier; no proxy fence: they only read it
+        // the buffer's last readers have passed a CTA barrier; no proxy fence: within a body's run
+        // ordinary accesses only read it (what came before is fenced at the run's start)
         mbar_expect_tx(bar, bytes);
         bulk_g2s(buf0 + (uint32_t)slot * bytes, a.coef + (size_t)blk(c) * Np, bytes, bar);
         issued = c + 1;
@@ -403,6 +404,9 @@ __device__ __forceinline__ void hvp_tma_body(const Args &a, int blk, unsigned ch
         for (int i = 0; i < S; ++i) mbar_init(ring.bar0 + 8u * i, 1);
         fence_mbar_init();
     }
+    // a batch kernel's earlier item, whose ring had another size, may have written these bytes as
+    // halo or state: order its ordinary accesses before the copies' writes
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     // behind the barrier: the flag is thread 0's store, and what the shared word held before it
     // (whatever an earlier kernel left) would end every wait of this thread at once
