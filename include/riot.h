@@ -318,8 +318,9 @@ riot_status riot_draw_normal(uint64_t seed, int64_t stream, int64_t n, int32_t n
 
 /* Standalone FP64 Lorenz-96 forecast: traj_dev ((T+1) x n doubles) gets the
  * RK4 trajectory from x0_dev, or only the final state when
- * store_all = 0 (traj_dev then holds n doubles).  Used to build synthetic
- * truths without a context. */
+ * store_all = 0 (traj_dev then holds n doubles).  x0_dev may lie anywhere in
+ * traj_dev, for instance be the last state of the forecast before.  Used to
+ * build synthetic truths without a context. */
 riot_status riot_l96_forecast(int64_t n, int32_t T, double dt, double F, const double *x0_dev,
                               double *traj_dev, int32_t store_all, void *cuda_stream);
 

@@ -91,7 +91,7 @@ struct L96Dev {
 };
 
 // Nonlinear FP64 trajectory of one state (l96_split.cu): traj (T+1)*n, or only the final
-// state into xT (which x0 must not alias) when traj is null, and the stage coefficients
+// state into xT when traj is null (x0 may lie anywhere in either), and the stage coefficients
 // (double2 by slot t*E + j; may be null; the padding slots of short chunks are not written).
 cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, double2 *coef64, double *xT, cudaStream_t s);
 // FP32 copy of the stage coefficients, interleaved by element pair ((j/2)*Tp + t as float4)

@@ -361,21 +361,25 @@ cudaError_t rows_zero(const L96Dev &m, cudaStream_t s)
 
 }  // namespace
 
-// The nonlinear trajectory from x0 (traj, or only the final state into xT) and its FP64 stage
-// coefficients (may be null).
+// The nonlinear trajectory from x0 (traj, or only the final state into xT; x0 may lie in either)
+// and its FP64 stage coefficients (may be null).
 cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, double2 *coef64, double *xT, cudaStream_t s)
 {
     const int n = m.geom.n, T = m.T;
-    if (T == 0)
-        return cudaMemcpyAsync(traj ? traj : xT, x0, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
     const SplitPlan pl = split_plan(n, 1);
-    // without a trajectory the states of successive launches alternate between xT and a
-    // temporary; a start that overlaps xT is set aside, since a launch's CTAs read it while others write
-    const bool clash = !traj && x0 < xT + n && xT < x0 + n, more = T > (pl.K > 0 ? pl.K : kMaxSteps);
+    // A launch's CTAs read the start while others write, so a start that overlaps what is written is
+    // set aside (one that is row 0 itself is only written with its own values).  Without a
+    // trajectory the states of successive launches alternate between xT and a temporary.
+    const double *end = traj ? traj + (size_t)(T + 1) * n : xT + n;
+    const bool clash = x0 != traj && x0 < end && (traj ? traj : xT) < x0 + n;
+    const bool more = !traj && T > (pl.K > 0 ? pl.K : kMaxSteps);
     double *tmp = nullptr;
     cudaError_t e;
-    if (!traj && (clash || more)) {
-        if ((e = cudaMallocAsync((void **)&tmp, 2 * sizeof(double) * n, s)) != cudaSuccess) return e;
+    if (clash || more) {
+        if ((e = cudaMallocAsync((void **)&tmp, 2 * sizeof(double) * n, s)) != cudaSuccess) {
+            cudaGetLastError();
+            return e;
+        }
         if (clash) {
             e = cudaMemcpyAsync(tmp + n, x0, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
             if (e != cudaSuccess) {
@@ -395,7 +399,8 @@ cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, doubl
     a.F = m.F;
     a.traj = traj;
     a.coef64 = coef64;
-    e = for_steps(pl, n, T, true, 1, nl_steps_kernel<true>, nl_steps_kernel<false>, a, s, [&](NlSteps &b, bool first) {
+    if (T == 0) e = x0 == traj ? cudaSuccess : cudaMemcpyAsync(traj ? traj : xT, x0, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
+    else e = for_steps(pl, n, T, true, 1, nl_steps_kernel<true>, nl_steps_kernel<false>, a, s, [&](NlSteps &b, bool first) {
         b.in = first ? x0 : traj ? traj + (size_t)b.t0 * n : prev;
         b.out = prev = ((launches - 1 - at++) & 1) ? tmp : xT;
     });
