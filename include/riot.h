@@ -30,11 +30,12 @@
  *    Eigenvalues are those of A (not I + A), sorted in decreasing order.
  *  - One context is not safe to use from two host threads at once.
  *  - Kernels with bounded device waits (the mixed-precision Hessian kernel's
- *    stage copies, the tensor-core GEMMs) never hang: a wait that runs out
- *    raises a flag and the kernel finishes with invalid results.  Every call
- *    that launches such kernels clears the flag when it starts and reads it
- *    before it returns (this synchronises), returning RIOT_ETIMEOUT; the
- *    context stays usable and the next call starts clean.
+ *    stage copies, the tensor-core GEMMs, the tridiagonal eigensolver's
+ *    barrier) never hang: a wait that runs out raises a flag and the kernel
+ *    finishes with invalid results.  Every call that launches such kernels
+ *    clears the flag when it starts and reads it before it returns (this
+ *    synchronises), returning RIOT_ETIMEOUT; the context stays usable and the
+ *    next call starts clean.
  */
 #ifndef RIOT_H
 #define RIOT_H
@@ -373,7 +374,8 @@ enum { RIOT_HVP_CTA_BARRIER = 0, RIOT_HVP_WARP_PAIRS = 1, RIOT_HVP_WARP_SHUFFLE 
 riot_status riot_set_hvp_kernel(riot_ctx *ctx, int32_t kernel);
 
 /* Bound of every wait of the mixed-precision Hessian kernels (on a stage copy,
- * or on a neighbouring warp's edge values), in tries of the waited mbarrier:
+ * or on a neighbouring warp's edge values), in tries of the waited mbarrier, and
+ * of the eigensolver's waits at its barrier (windows of a batch keep the default):
  * polls >= 0 sets it (0 gives up at once, so the next Hessian application
  * reports RIOT_ETIMEOUT without a fault: this is how the timeout report is
  * tested), polls < 0 restores the default (a wait gives up after well under a

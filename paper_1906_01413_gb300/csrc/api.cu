@@ -41,7 +41,7 @@ struct riot_ctx {
     riot_dev_free_fn dev_free = nullptr;
     void *alloc_user = nullptr;
     std::vector<riot_alloc_rec> allocs;
-    int wait_polls = -1;   // poll bound of the Hessian kernel's waits (-1: default; riot_set_wait_limit)
+    int wait_polls = -1;   // poll bound of the Hessian kernel's and the eigensolver's waits (-1: default; riot_set_wait_limit)
     // model tables
     int *optr = nullptr, *oslot = nullptr, *oidx = nullptr;
     double *y = nullptr, *rinv64 = nullptr, *band64 = nullptr, *sig64 = nullptr;
@@ -372,7 +372,8 @@ riot_status check_cholesky(riot_ctx *ctx, int base, int count, const char *what)
 }
 
 // The flag of the kernels with bounded device waits (the mixed-precision Hessian
-// kernel's stage copies, the tensor-core GEMMs' MMA completions): every call that
+// kernel's stage copies, the tensor-core GEMMs' MMA completions, the
+// tridiagonalisation's barrier): every call that
 // launches them clears it first and reads it (synchronising) before it returns, so
 // each call reports its own timeout and a later call is not blamed for it.
 riot_status clear_timeout(riot_ctx *ctx)
@@ -393,8 +394,8 @@ riot_status check_timeout(riot_ctx *ctx)
                     "a bounded device wait ran out and a bulk copy was still in flight when its CTA exited: every "
                     "result of that launch is invalid");
     return fail(ctx, RIOT_ETIMEOUT,
-                "a bounded device wait ran out (Hessian kernel stage copy or tensor-core GEMM): the results of this "
-                "call are invalid");
+                "a bounded device wait ran out (Hessian kernel stage copy, tensor-core GEMM or the eigensolver's barrier): "
+                "the results of this call are invalid");
 }
 
 // ---------------------------------------------------------------------------
@@ -1125,7 +1126,7 @@ riot_status rsvd_eig(riot_ctx *ctx, int k)
         CU(jacobi_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->s));
     else
         CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, ctx->s,
-                       ctx->prec == RIOT_PREC_MIXED, ctx->prec == RIOT_PREC_MIXED ? ctx->errflag : nullptr));
+                       ctx->prec == RIOT_PREC_MIXED, ctx->prec == RIOT_PREC_MIXED ? ctx->errflag : nullptr, ctx->wait_polls));
     if (ctx->scale_exp) CU(scal(k, ldexp(1.0, ctx->scale_exp), ctx->lam, ctx->s));
     return RIOT_OK;
 }
@@ -2482,7 +2483,8 @@ static riot_status varcg_body(riot_ctx *ctx, int32_t m, double *dv_dev, double *
     // T_m, its eigenpairs (theta, Z), U = Q Z, dv = -U diag(1 / (1 + theta)) U^T g
     CU(cudaMemcpyAsync(betas_dev, betas.data(), sizeof(double) * mm, cudaMemcpyHostToDevice, s));
     CU(tridiag_fill(mm, alphas, betas_dev, ctx->Km, s));
-    CU(tridiag_eig(ctx->Km, mm, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s));
+    CU(tridiag_eig(ctx->Km, mm, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s, false, nullptr,
+                   ctx->wait_polls));
     int einfo[2] = {0, 0};
     CU(cudaMemcpyAsync(einfo, ctx->info + 12, sizeof(einfo), cudaMemcpyDeviceToHost, s));
     CU(cudaStreamSynchronize(s));
@@ -2506,14 +2508,16 @@ static riot_status varcg_body(riot_ctx *ctx, int32_t m, double *dv_dev, double *
 
 // Eigenpairs of the k x k matrix in Km (not modified by the tridiagonal solver) into lam, Z:
 // the tridiagonal solver, and Jacobi when close eigenvalues left inverse iteration with
-// dependent vectors.  Synchronises.
+// dependent vectors.  Synchronises, and reports a wait that ran out since the flag was cleared, so
+// that nothing is formed from pairs that are wrong.
 static riot_status small_eig(riot_ctx *ctx, int k, const char *what)
 {
     cudaStream_t s = ctx->s;
-    CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s));
+    CU(tridiag_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, ctx->errflag, s, false, nullptr,
+                   ctx->wait_polls));
     int einfo[2] = {0, 0};
     CU(cudaMemcpyAsync(einfo, ctx->info + 12, sizeof(einfo), cudaMemcpyDeviceToHost, s));
-    CU(cudaStreamSynchronize(s));
+    TRY(check_timeout(ctx));   // synchronises
     if (einfo[0] || einfo[1]) {
         CU(jacobi_eig(ctx->Km, k, ctx->lam, ctx->Z, ctx->jwork, ctx->info + 12, s));
         CU(cudaMemcpyAsync(einfo, ctx->info + 12, sizeof(einfo), cudaMemcpyDeviceToHost, s));
@@ -2699,6 +2703,7 @@ riot_status riot_psas(riot_ctx *ctx, int32_t m, int32_t q, int64_t sketch_stream
     if (!ctx->pc_m.empty()) return fail(ctx, RIOT_ESTATE, "riot_psas: Algorithm 4 runs without the spectral preconditioner");
     CU(cudaSetDevice(ctx->dev));
     TRY(psas_alloc(ctx));
+    TRY(clear_timeout(ctx));   // read by small_eig, before x and v change
     const int n = ctx->n, p = ctx->p;
     cudaStream_t s = ctx->s;
     ctx->have_rsvd = 0;   // the primal Ritz pairs are not kept

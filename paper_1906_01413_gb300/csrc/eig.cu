@@ -359,14 +359,14 @@ struct TridiagProb {
     double *A, *Qt, *pq, *d, *e;
     unsigned *bar;   // zero at launch
     int *err;        // raised if a wait at the barrier ran out
-    int k, cta0, G;
+    int k, cta0, G, polls;
 };
 constexpr int kTridiagProbs = 48;
 struct TridiagProbs {
     TridiagProb p[kTridiagProbs];
     int n;
 };
-constexpr int kBarrierPolls = 1 << 20;   // about half a second
+constexpr int kBarrierPolls = 1 << 20;   // default bound of a wait: about half a second
 
 __global__ void __launch_bounds__(256) tridiag_group_kernel(const __grid_constant__ TridiagProbs a)
 {
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(256) tridiag_group_kernel(const __grid_constan
             for (int t = 0; !dead; ++t) {
                 asm volatile("ld.acquire.gpu.u32 %0, [%1];" : "=r"(seen) : "l"(p.bar) : "memory");
                 if (seen >= target) break;
-                if (t == kBarrierPolls) {
+                if (t == p.polls) {
                     dead = true;   // later waits return at once; the result is wrong and flagged
                     atomicMax(p.err, 1);
                 }
@@ -1026,7 +1026,7 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
             const int G = (j.k + 3) / 4;
             if (a.n > 0 && ctas + G > room) break;
             const EigWork w(j.work, j.k);
-            a.p[a.n++] = {w.A, w.Qt, w.pq, w.d, w.e, w.bar, j.err, j.k, ctas, G};
+            a.p[a.n++] = {w.A, w.Qt, w.pq, w.d, w.e, w.bar, j.err, j.k, ctas, G, j.polls < 0 ? kBarrierPolls : j.polls};
             ctas += G;
             ++at;
         }
@@ -1040,10 +1040,10 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
 }
 
 cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, int *err, cudaStream_t s,
-                        bool fp32_vectors, int *tc_err)
+                        bool fp32_vectors, int *tc_err, int wait_polls)
 {
     cudaError_t e = tridiag_prepare(K, k, work, info, s);
-    const TridiagJob job = {k, work, err};
+    const TridiagJob job = {k, work, err, wait_polls};
     if (e == cudaSuccess) e = tridiag_run(&job, 1, s);
     return e == cudaSuccess ? tridiag_finish(k, lam, Z, work, info, s, fp32_vectors, tc_err, true) : e;
 }

@@ -345,9 +345,10 @@ size_t jacobi_work_doubles(int k);
 // stops at about 1e-7 (one shifted CholeskyQR pass less); with tc_err (the flag of the
 // tensor-core kernels' bounded waits) it runs on their FP32 rounding with the exact
 // tensor-core Gram and the one-launch FP32 solve, as the mixed path's CholeskyQR does
-// err: raised if a wait at the tridiagonalisation's barrier ran out.
+// err: raised if a wait at the tridiagonalisation's barrier ran out, after wait_polls tries (< 0: the
+// default, well under a second).
 cudaError_t tridiag_eig(const double *K, int k, double *lam, double *Z, double *work, int *info, int *err, cudaStream_t s,
-                        bool fp32_vectors = false, int *tc_err = nullptr);
+                        bool fp32_vectors = false, int *tc_err = nullptr, int wait_polls = -1);
 // The same in three parts, so that several problems tridiagonalise side by side in one
 // cooperative launch: prepare, run and finish on each problem's workspace; prepare and finish may
 // be on parallel streams (whole_gpu false then, as for cholesky).
@@ -355,6 +356,7 @@ struct TridiagJob {
     int k;
     double *work;
     int *err;
+    int polls = -1;
 };
 cudaError_t tridiag_prepare(const double *K, int k, double *work, int *info, cudaStream_t s);
 cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s);

@@ -289,7 +289,8 @@ def riot_set_hvp_kernel(ctx, kernel):
 
 
 def riot_set_wait_limit(ctx, polls):
-    """Poll bound of the Hessian kernel's waits (< 0: the default); tests of the timeout report."""
+    """Poll bound of the Hessian kernel's and the eigensolver's waits (< 0: the default); tests of the
+    timeout report."""
     _check(ctx, "riot_set_wait_limit", load().riot_set_wait_limit(ctx, int(polls)))
 
 
