@@ -138,23 +138,105 @@ cudaError_t conv(const float *in, int ci, const float *W, const float *bias, con
 
 // Weight gradient: gW[o][c][d] = sum_b sum_i gout[b][o][i] in[b][c][(i + d - h) mod n], gb[o] =
 // sum gout, to the accuracy of sums in 64 bits.  FP64 is 1/64 of the FP32 rate here, so each sum
-// is a compensated FP32 one (after Ogita, Rump and Oishi 2005: the rounding error of every step
-// is added to a second FP32 word): 4 FP32 operations a term against 64 issue slots.  A warp owns 4 output channels x 1 input channel x K taps, lanes run
-// over positions; 20 sums (K = 5) share 9 loads.  Lanes' and slots' sums are then added in FP64.
-// A sum that is not finite is formed again in FP64 (a product may leave the FP32 range).
-// Bound: FP32 issue and load latency (24 warps an SM: 80 registers; at 152 registers and 8 warps it
-// takes 1.8 times as long).  n = 4096, batch 8: 64 x 64 channels 225 us, all layers 12.2 -> 0.93 ms,
-// the gradient's error 6.6e-7 -> 4.6e-7 (that of the FP32 factors).
-constexpr int kGradO = 4, kGradU = 2;
+// is a compensated FP32 one, the dot product in twice the working precision of Ogita, Rump and
+// Oishi 2005 (Dot2): 10 FP32 operations a term, packed for two outputs, against 64 issue slots.  A
+// warp owns 4 output channels x 1 input channel x K taps, lanes run over positions; 20 sums (K = 5)
+// share 9 loads.  Slots' sums are then added in FP64.  A sum that is not finite (a product may
+// leave the FP32 range) or so small that the rounding errors of its products may be below that
+// range is formed again in FP64.
+// Bound: FP32 issue (77 % of the slots with unpacked operations, 2.20 ms a training batch; packed
+// 2.07), 16 warps an SM for the loads of 4 positions in flight (24 warps with 2: 2.23 ms).  n = 4096,
+// batch 8, 8 - 64 - 64 - 64 - 128 channels: FP64 sums 12.2 ms, this 1.18 ms, the same gradient error
+// (6.8e-7, that of the FP32 factors).  Fast2Sum without its ordering, 4 operations a term, took
+// 0.93 ms and was off by 6 % where a lane's terms cancel to 2^-21.
+constexpr int kGradO = 4;
 
-// s + g x rounded, what the rounding lost added to c.  s - t is exact while the sum is at least as
-// large as the term (Fast2Sum); otherwise its rounding is 2^-25 of the term, once.
-__device__ __forceinline__ void dot2(float g, float x, float &s, float &c)
+// s + g x, what its product and its sum lose added to c.  Both losses are exact whatever the sizes of
+// s and g x (products above 2^-102): where terms cancel, the sum is smaller than a term.
+struct Two {
+    float s, c;
+};
+__device__ __forceinline__ float sum2(float &s, float p)   // the loss of s += p
 {
-    const float t = __fmaf_rn(g, x, s);
-    c = __fadd_rn(c, __fmaf_rn(g, x, __fsub_rn(s, t)));
+    const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+    const float lost = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z));
     s = t;
+    return lost;
 }
+// The same of two sums side by side, in packed instructions: s + g x, ng = -g.
+using pair_t = unsigned long long;
+struct Two2 {
+    pair_t s, c;
+};
+__device__ __forceinline__ pair_t pk(float x, float y)
+{
+    pair_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 upk(pair_t p)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ pair_t add_pair(pair_t a, pair_t b)
+{
+    pair_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ pair_t sub_pair(pair_t a, pair_t b)
+{
+    pair_t r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ void dot2(pair_t g, pair_t ng, pair_t x, Two2 &v)
+{
+    pair_t p, low;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(p) : "l"(g), "l"(x));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(low) : "l"(ng), "l"(x), "l"(p));   // what p has too much
+    const pair_t t = add_pair(v.s, p), z = sub_pair(t, v.s);
+    const pair_t lost = add_pair(sub_pair(v.s, sub_pair(t, z)), sub_pair(p, z));
+    v.c = add_pair(v.c, sub_pair(lost, low));
+    v.s = t;
+}
+__device__ __forceinline__ Two added(Two a, Two b)
+{
+    const float lost = sum2(a.s, b.s);
+    return {a.s, __fadd_rn(__fadd_rn(a.c, b.c), lost)};
+}
+__device__ __forceinline__ double added(double a, double b) { return a + b; }
+__device__ __forceinline__ double across(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
+__device__ __forceinline__ Two across(Two v, int off)
+{
+    return {__shfl_xor_sync(0xffffffffu, v.s, off), __shfl_xor_sync(0xffffffffu, v.c, off)};
+}
+
+// Sums over the lanes, lane j ending with sum j: each exchange halves the sums a lane carries.
+template <int NV, typename T>
+__device__ __forceinline__ T lane_sums(T (&v)[NV])
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool up = threadIdx.x & off;
+#pragma unroll
+        for (int j = 0; j < off && j < NV; ++j) {
+            if (j + off < NV) {
+                const T lo = v[j], hi = v[j + off < NV ? j + off : 0];
+                v[j] = added(up ? hi : lo, across(up ? lo : hi, off));
+            } else {
+                v[j] = added(v[j], across(v[j], off));
+            }
+        }
+    }
+    return v[0];
+}
+
+// A warp's sum of fewer than 2^20 terms above this lost less than 2^-30 of itself to products whose
+// rounding error is below the smallest FP32 number.
+constexpr double kTinySum = 7.8886e-31;   // 2^-100
 
 // What one warp adds up: positions lo, lo + 1, .. of the units (window, range) of its slot.
 struct GradWork {
@@ -165,7 +247,7 @@ struct GradWork {
 template <int K, typename F>
 __device__ __forceinline__ void wgrad_sweep(const GradWork &a, F add)
 {
-    constexpr int h = K / 2;
+    constexpr int h = K / 2, kGradU = K <= 5 ? 4 : 2;   // positions whose loads are in flight together
     const int lane = threadIdx.x & 31, n = a.n;
     const int len = ((n + a.csplit - 1) / a.csplit + 31) / 32 * 32;   // positions of a unit
     for (int u = blockIdx.z; u < a.B * a.csplit; u += gridDim.z) {
@@ -203,7 +285,7 @@ __device__ __forceinline__ void wgrad_sweep(const GradWork &a, F add)
 }
 
 template <int K>
-__global__ void __launch_bounds__(256, 3) conv_wgrad_kernel(const float *gout, int co, const float *in, int ci, int n,
+__global__ void __launch_bounds__(256, 2) conv_wgrad_kernel(const float *gout, int co, const float *in, int ci, int n,
                                                             int B, int csplit, double *part)
 {
     constexpr int NV = kGradO * K;
@@ -211,65 +293,91 @@ __global__ void __launch_bounds__(256, 3) conv_wgrad_kernel(const float *gout, i
     const int o0 = (blockIdx.x * 2 + (wp >> 2)) * kGradO, c = blockIdx.y * 4 + (wp & 3);
     if (o0 >= co || c >= ci) return;
     const GradWork a = {gout, in, co, ci, n, B, csplit, o0, c};
-    double v[32], vb[kGradO];
-    bool bad = false;
-    {
-        float s[NV], e[NV], sb[kGradO], eb[kGradO];
-#pragma unroll
-        for (int j = 0; j < NV; ++j) s[j] = e[j] = 0.f;
-#pragma unroll
-        for (int q = 0; q < kGradO; ++q) sb[q] = eb[q] = 0.f;
-        wgrad_sweep<K>(a, [&](const float(&g)[kGradO], const float(&x)[K]) {
-#pragma unroll
-            for (int q = 0; q < kGradO; ++q) {
-#pragma unroll
-                for (int d = 0; d < K; ++d) dot2(g[q], x[d], s[q * K + d], e[q * K + d]);
-                if (c == 0) dot2(g[q], 1.f, sb[q], eb[q]);
-            }
-        });
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            v[j] = j < NV ? (double)s[j < NV ? j : 0] + (double)e[j < NV ? j : 0] : 0.0;
-            if (j < NV) bad |= !isfinite(s[j < NV ? j : 0] + e[j < NV ? j : 0]);
-        }
-#pragma unroll
-        for (int q = 0; q < kGradO; ++q) {
-            vb[q] = (double)sb[q] + (double)eb[q];
-            bad |= !isfinite(sb[q] + eb[q]);
-        }
-    }
-    if (__any_sync(0xffffffffu, bad)) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = 0.0;
-#pragma unroll
-        for (int q = 0; q < kGradO; ++q) vb[q] = 0.0;
-        wgrad_sweep<K>(a, [&](const float(&g)[kGradO], const float(&x)[K]) {
-#pragma unroll
-            for (int q = 0; q < kGradO; ++q) {
-#pragma unroll
-                for (int d = 0; d < K; ++d) v[q * K + d] = fma((double)g[q], (double)x[d], v[q * K + d]);
-                vb[q] += g[q];
-            }
-        });
-    }
-    // add over the lanes, lane j ending with sum j: each exchange halves the sums a lane carries
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-        for (int j = 0; j < off; ++j) {
-            const bool up = lane & off;
-            const double mine = up ? v[j + off] : v[j], give = up ? v[j] : v[j + off];
-            v[j] = mine + __shfl_xor_sync(0xffffffffu, give, off);
-        }
-    double *out = part + (size_t)blockIdx.z * ((size_t)co * ci * K + co);
     const int q = lane / K, d = lane - q * K;
-    if (lane < NV && o0 + q < co) out[((size_t)(o0 + q) * ci + c) * K + d] = v[0];
+    const bool mine = lane < NV && o0 + q < co;
+    double v = 0.0, vb[kGradO];   // sum `lane` of the weights, the sums of the biases
+    for (bool again = false;; again = true) {
+        if (!again) {
+            Two u[NV], ub[kGradO];
+            Two2 w[kGradO / 2][K];
+#pragma unroll
+            for (int r = 0; r < kGradO / 2; ++r)
+#pragma unroll
+                for (int j = 0; j < K; ++j) w[r][j] = {0, 0};
+#pragma unroll
+            for (int r = 0; r < kGradO; ++r) ub[r] = {0.f, 0.f};
+            wgrad_sweep<K>(a, [&](const float(&g)[kGradO], const float(&x)[K]) {
+#pragma unroll
+                for (int r = 0; r < kGradO / 2; ++r) {
+                    const pair_t gp = pk(g[2 * r], g[2 * r + 1]), ng = pk(-g[2 * r], -g[2 * r + 1]);
+#pragma unroll
+                    for (int j = 0; j < K; ++j) dot2(gp, ng, pk(x[j], x[j]), w[r][j]);
+                }
+                if (c == 0)
+#pragma unroll
+                    for (int r = 0; r < kGradO; ++r) ub[r].c = __fadd_rn(ub[r].c, sum2(ub[r].s, g[r]));
+            });
+#pragma unroll
+            for (int r = 0; r < kGradO / 2; ++r)
+#pragma unroll
+                for (int j = 0; j < K; ++j) {
+                    const float2 s2 = upk(w[r][j].s), c2 = upk(w[r][j].c);
+                    u[2 * r * K + j] = {s2.x, c2.x};
+                    u[(2 * r + 1) * K + j] = {s2.y, c2.y};
+                }
+            const Two t = lane_sums<NV>(u);
+            v = (double)t.s + (double)t.c;
+            if (c == 0)
+#pragma unroll
+                for (int r = 0; r < kGradO; ++r) {
+                    for (int off = 16; off > 0; off >>= 1) ub[r] = added(ub[r], across(ub[r], off));
+                    vb[r] = (double)ub[r].s + (double)ub[r].c;
+                }
+        } else {
+            double u[NV];
+#pragma unroll
+            for (int j = 0; j < NV; ++j) u[j] = 0.0;
+#pragma unroll
+            for (int r = 0; r < kGradO; ++r) vb[r] = 0.0;
+            wgrad_sweep<K>(a, [&](const float(&g)[kGradO], const float(&x)[K]) {
+#pragma unroll
+                for (int r = 0; r < kGradO; ++r) {
+#pragma unroll
+                    for (int j = 0; j < K; ++j) u[r * K + j] = fma((double)g[r], (double)x[j], u[r * K + j]);
+                    vb[r] += g[r];
+                }
+            });
+            v = lane_sums<NV>(u);
+            if (c == 0)
+#pragma unroll
+                for (int r = 0; r < kGradO; ++r)
+                    for (int off = 16; off > 0; off >>= 1) vb[r] += across(vb[r], off);
+        }
+        if (again) break;
+        bool bad = mine && !isfinite(v);
+        if (c == 0)
+#pragma unroll
+            for (int r = 0; r < kGradO; ++r) bad |= !isfinite(vb[r]);
+        if (__any_sync(0xffffffffu, bad)) continue;
+        if (!__any_sync(0xffffffffu, mine && fabs(v) < kTinySum)) break;
+        // tiny sums of zeros are right: does one have factors?
+        unsigned gs = 0, xs = 0;   // bit r: gradient of output r, bit 0: input
+        wgrad_sweep<K>(a, [&](const float(&g)[kGradO], const float(&x)[K]) {
+#pragma unroll
+            for (int r = 0; r < kGradO; ++r) gs |= (g[r] != 0.f) << r;
+#pragma unroll
+            for (int j = 0; j < K; ++j) xs |= x[j] != 0.f;
+        });
+        gs = __reduce_or_sync(0xffffffffu, gs);
+        xs = __reduce_or_sync(0xffffffffu, xs);
+        if (!xs || !__any_sync(0xffffffffu, mine && fabs(v) < kTinySum && ((gs >> q) & 1))) break;
+    }
+    double *out = part + (size_t)blockIdx.z * ((size_t)co * ci * K + co);
+    if (mine) out[((size_t)(o0 + q) * ci + c) * K + d] = v;
     if (c == 0)
 #pragma unroll
-        for (int r = 0; r < kGradO; ++r) {
-            for (int off = 16; off > 0; off >>= 1) vb[r] += __shfl_xor_sync(0xffffffffu, vb[r], off);
+        for (int r = 0; r < kGradO; ++r)
             if (lane == 0 && o0 + r < co) out[(size_t)co * ci * K + o0 + r] = vb[r];
-        }
 }
 
 __global__ void wgrad_sum_kernel(const double *part, int slots, size_t count, float *grad)
