@@ -837,7 +837,7 @@ riot_status setup_common(riot_ctx *ctx)
         (st = dalloc(ctx, &ctx->dv, np)) || (st = dalloc(ctx, &ctx->tmp, np)) || (st = dalloc(ctx, &ctx->d, p)) ||
         (st = dalloc(ctx, &ctx->v0, np)) ||
         (st = dalloc(ctx, &ctx->xsave, np)) || (st = dalloc(ctx, &ctx->vsave, np)) ||
-        (st = dalloc(ctx, &ctx->rd, p)) || (st = dalloc(ctx, &ctx->jo, 2)) ||
+        (st = dalloc(ctx, &ctx->rd, p)) || (st = dalloc(ctx, &ctx->jo, kJoDoubles)) ||
         (st = dalloc(ctx, (char **)&ctx->Wblk, np * k * rs)) || (st = dalloc(ctx, (char **)&ctx->Yblk, np * k * rs)) ||
         (st = dalloc(ctx, &ctx->Q, np * k)) || (st = dalloc(ctx, &ctx->U, np * k)) ||
         (ctx->prec == RIOT_PREC_MIXED &&

@@ -96,8 +96,10 @@ struct L96Dev {
 cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, double2 *coef64, double *xT, cudaStream_t s);
 // FP32 copy of the stage coefficients, interleaved by element pair ((j/2)*Tp + t as float4)
 cudaError_t l96_coef32(const L96Dev &m, const double2 *coef64, float2 *coef32, cudaStream_t s);
-// The innovation d = H(x) - y from the trajectory and 1/2 sum d^2/sigma^2 added to *jo; with
-// rows, R^-1 d becomes the forcing of l96_split_gradient (needs the split workspace).
+// The innovation d = H(x) - y from the trajectory and 1/2 sum d^2/sigma^2 added to jo[0]; jo has
+// kJoDoubles, of which the first two are zero at the call and the others scratch.  With rows,
+// R^-1 d becomes the forcing of l96_split_gradient (needs the split workspace).
+constexpr int kJoDoubles = 2 + 256;
 cudaError_t l96_innov(const L96Dev &m, const double *traj, double *d, double *jo, bool rows, cudaStream_t s);
 // b = L^T H^T R^-1 d after l96_innov(rows), and y = A z when z is given (sp.cols >= 2 then)
 cudaError_t l96_split_gradient(const L96Dev &m, const double2 *coef, double *b, const double *z, double *y,

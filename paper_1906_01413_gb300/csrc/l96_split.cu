@@ -244,11 +244,29 @@ __global__ void __launch_bounds__(512) ad_steps_kernel(const LinSteps a)
     a.out[(size_t)blockIdx.y * a.lds + p.i] = lam;
 }
 
-// d = H(x) - y, 1/2 sum d^2 / sigma^2, and R^-1 d added to the rows (zeroed before)
+constexpr int kInnovCtas = kJoDoubles - 2;   // a partial sum each
+
+// The sum of a value per thread of a CTA of 256, in a fixed order; thread 0 has it.
+__device__ __forceinline__ double cta_sum(double s)
+{
+    __shared__ double ws[8];
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < 8; ++w) s += ws[w];
+    return s;
+}
+
+// d = H(x) - y, 1/2 sum d^2 / sigma^2 added to jo[0], and R^-1 d added to the rows (zeroed before).
+// The sum is the same bits every time: the CTAs' partial sums (jo[2] on) are added in order by the
+// CTA that finishes last (counted in the bytes of jo[1], zero at launch).
 __global__ void __launch_bounds__(256) innov_kernel(int p, int n, const int *obsrow, const int *rowstep, const int *oidx,
                                                     const double *traj, const double *y, const double *rinv, double *d,
                                                     double *rows, double *jo)
 {
+    __shared__ bool last;
     double s = 0.0;
     for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < p; o += gridDim.x * blockDim.x) {
         const int r = obsrow[o], i = oidx[o];
@@ -257,8 +275,17 @@ __global__ void __launch_bounds__(256) innov_kernel(int p, int n, const int *obs
         if (rows) atomicAdd(&rows[(size_t)r * n + i], w);
         s = fma(0.5 * dd, w, s);
     }
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0 && s != 0.0) atomicAdd(jo, s);
+    s = cta_sum(s);
+    if (threadIdx.x == 0) {
+        jo[2 + blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd((unsigned *)(jo + 1), 1u) + 1 == gridDim.x;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    s = cta_sum(threadIdx.x < gridDim.x ? __ldcg(jo + 2 + threadIdx.x) : 0.0);
+    if (threadIdx.x == 0) jo[0] += s;
 }
 
 __global__ void rows_scatter_kernel(int p, int n, const int *obsrow, const int *oidx, const double *r, double *rows)
@@ -529,7 +556,7 @@ cudaError_t l96_innov(const L96Dev &m, const double *traj, double *d, double *jo
     if (m.p == 0) return cudaSuccess;
     cudaError_t e;
     if (rows && (e = rows_zero(m, s)) != cudaSuccess) return e;
-    const unsigned grid = blocks_for(m.p, 256) < 256 ? blocks_for(m.p, 256) : 256;
+    const unsigned grid = blocks_for(m.p, 256) < kInnovCtas ? blocks_for(m.p, 256) : kInnovCtas;
     count_launch();
     innov_kernel<<<grid, 256, 0, s>>>(m.p, m.geom.n, m.sp.obsrow, m.sp.rowstep, m.oidx, traj, m.y, m.rinv64, d,
                                       rows ? m.sp.rows : nullptr, jo);
