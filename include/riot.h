@@ -178,10 +178,13 @@ typedef struct riot_ctx riot_ctx;
  * observations and the B descriptor to the device, builds L, and allocates
  * all workspace for kmax sketch columns (through opt->dev_alloc when given;
  * a NULL from it is RIOT_ENOMEM, a pointer not aligned to 256 bytes
- * RIOT_EINVAL; only the Lorenz-96 workspace that lets FP64 integrations of a
- * few columns spread over the GPU may be refused: they then run slower).  It also looks up, once per device, the device address of
- * the static scratch array of riot_hessian_apply_noalloc.  cuda_stream is a
- * cudaStream_t (NULL = legacy default stream).  On failure *out is NULL. */
+ * RIOT_EINVAL).  Asked for last, a Lorenz-96 workspace that lets FP64
+ * integrations of a few columns spread over the GPU (24 bytes per variable and
+ * observed step, or up to 256 MB more) may be refused, and is given back when a
+ * later allocation of the context fails: they then run slower.  The call also
+ * looks up, once per device, the device address of the static scratch array of
+ * riot_hessian_apply_noalloc.  cuda_stream is a cudaStream_t (NULL = legacy
+ * default stream).  On failure *out is NULL. */
 riot_status riot_setup(riot_ctx **out, const riot_model_desc *model, const riot_obs_desc *obs,
                        const riot_bcov_desc *B, const riot_options *opt, void *cuda_stream);
 

@@ -41,6 +41,7 @@ struct riot_ctx {
     riot_dev_free_fn dev_free = nullptr;
     void *alloc_user = nullptr;
     std::vector<riot_alloc_rec> allocs;
+    riot_alloc_rec split_ws = {nullptr, 0};   // workspace of the split FP64 integrations (setup_split), optional
     int wait_polls = -1;   // poll bound of the Hessian kernel's and the eigensolver's waits (-1: default; riot_set_wait_limit)
     // model tables
     int *optr = nullptr, *oslot = nullptr, *oidx = nullptr;
@@ -167,24 +168,32 @@ riot_status fail(riot_ctx *c, riot_status st, const char *fmt, ...)
         if (e_ != cudaSuccess) return bfail(b, RIOT_ECUDA, "%s failed: %s", #call, cudaGetErrorString(e_)); \
     } while (0)
 
-// Device memory of a context: from the caller's allocator when riot_options gave one,
-// else cudaMalloc.  Returns NULL on failure.
-void *ctx_malloc(riot_ctx *ctx, size_t bytes)
-{
-    if (ctx->dev_alloc) return ctx->dev_alloc(bytes, (void *)ctx->s, ctx->alloc_user);
-    void *q = nullptr;
-    if (cudaMalloc(&q, bytes) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return q;
-}
-
 void ctx_free(riot_ctx *ctx, const riot_alloc_rec &a)
 {
     if (!a.p) return;
     if (ctx->dev_free) ctx->dev_free(a.p, a.bytes, (void *)ctx->s, ctx->alloc_user);
     else cudaFree(a.p);
+}
+
+// Device memory of a context: from the caller's allocator when riot_options gave one,
+// else cudaMalloc.  The optional workspace (setup_split) is given back when it stands in the
+// way of anything else.  Returns NULL on failure.
+void *ctx_malloc(riot_ctx *ctx, size_t bytes)
+{
+    for (;;) {
+        void *q = nullptr;
+        if (ctx->dev_alloc) {
+            q = ctx->dev_alloc(bytes, (void *)ctx->s, ctx->alloc_user);
+        } else if (cudaMalloc(&q, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            q = nullptr;
+        }
+        if (q || !ctx->split_ws.p) return q;
+        cudaStreamSynchronize(ctx->s);   // queued integrations may still use it
+        ctx_free(ctx, ctx->split_ws);
+        ctx->split_ws = {nullptr, 0};
+        ctx->m.sp.drop();
+    }
 }
 
 template <typename T>
@@ -502,14 +511,11 @@ void sym_sqrt_host(std::vector<double> &A, int n)
         }
 }
 
-// Tables of the split FP64 integrations and, when memory allows, their workspace: room for a
-// few columns (rows of the observed steps and two states each, 256 MB at most beyond
-// two).  Without it (the allocator returned NULL) those integrations take one CTA a column.
-riot_status setup_split(riot_ctx *ctx, const std::vector<int> &optr, const std::vector<int> &oidx,
-                        const std::vector<double> &rinv)
+// Tables of the FP64 integrations' observed steps.
+riot_status setup_obs_rows(riot_ctx *ctx, const std::vector<int> &optr)
 {
     L96Dev &m = ctx->m;
-    const int n = ctx->n, p = ctx->p, T = m.T;
+    const int p = ctx->p, T = m.T;
     std::vector<int> orow(T + 1, -1), rowstep, obsrow(p);
     for (int t = 0; t <= T; ++t)
         if (optr[t] < optr[t + 1]) {
@@ -517,38 +523,54 @@ riot_status setup_split(riot_ctx *ctx, const std::vector<int> &optr, const std::
             rowstep.push_back(t);
             for (int j = optr[t]; j < optr[t + 1]; ++j) obsrow[j] = orow[t];
         }
-    const size_t nrow = rowstep.size(), np = (size_t)n, col = (nrow + 2) * np;
-    m.sp.nrow = (int)nrow;
-    m.sp.last_step = nrow ? rowstep.back() : -1;
+    m.sp.nrow = (int)rowstep.size();
+    m.sp.last_step = rowstep.empty() ? -1 : rowstep.back();
     int *d_rowstep = nullptr, *d_obsrow = nullptr;
-    TRY(dalloc(ctx, &d_rowstep, nrow));
+    TRY(dalloc(ctx, &d_rowstep, rowstep.size()));
     TRY(dalloc(ctx, &d_obsrow, (size_t)p));
     m.sp.orow_h = orow;
     m.sp.rowstep = d_rowstep;
     m.sp.obsrow = d_obsrow;
+    cudaError_t e = cudaSuccess;
+    if ((e = up(ctx, d_rowstep, rowstep.data(), rowstep.size())) ||
+        (e = up(ctx, d_obsrow, obsrow.data(), obsrow.size())) || (e = cudaStreamSynchronize(ctx->s)))
+        return fail(ctx, RIOT_ECUDA, "setup upload failed: %s", cudaGetErrorString(e));
+    return RIOT_OK;
+}
+
+// The workspace of the split FP64 integrations, when memory allows (asked for after everything
+// else): the weights of the observed steps' rows and room for a few columns, rows and two states
+// each, 256 MB of them at most but always two (the gradient and the product that scales the FP32
+// path; with the weights 24 bytes per variable and observed step, a quarter of the trajectory and its
+// coefficients at most).  Without it those integrations take one CTA a column.
+riot_status setup_split(riot_ctx *ctx, const riot_obs_desc *obs)
+{
+    L96Dev &m = ctx->m;
+    const size_t nrow = (size_t)m.sp.nrow, np = (size_t)ctx->n, col = (nrow + 2) * np;
     size_t cols = ((size_t)256 << 20) / (col * sizeof(double));
     cols = cols > 16 ? 16 : cols;
     if (cols > (size_t)ctx->kmax) cols = (size_t)ctx->kmax;
-    if (cols < 2) cols = 2;   // the gradient and the product that scales the FP32 path
-    double *wgt = nullptr, *work = nullptr;
-    riot_status st = dalloc(ctx, &wgt, nrow * np);
-    if (st == RIOT_OK) st = dalloc(ctx, &work, cols * col);
-    if (st != RIOT_OK && st != RIOT_ENOMEM) return st;
-    std::vector<double> w;
-    cudaError_t e = cudaSuccess;
-    if (st == RIOT_OK) {
-        w.assign(nrow * np, 0.0);
-        for (int j = 0; j < p; ++j) w[(size_t)obsrow[j] * np + oidx[j]] += rinv[j];
-        e = up(ctx, wgt, w.data(), w.size());
-        m.sp.wgt = wgt;
-        m.sp.rows = work;
-        m.sp.a = work + cols * nrow * np;
-        m.sp.b = m.sp.a + cols * np;
-        m.sp.cols = (int)cols;
+    if (cols < 2) cols = 2;
+    double *work = nullptr;
+    const riot_status st = dalloc(ctx, &work, nrow * np + cols * col);
+    if (st == RIOT_ENOMEM) {
+        ctx->err[0] = 0;   // not a failure of the call
+        return RIOT_OK;
     }
-    if (e || (e = up(ctx, d_rowstep, rowstep.data(), nrow)) ||
-        (e = up(ctx, d_obsrow, obsrow.data(), obsrow.size())) || (e = cudaStreamSynchronize(ctx->s)))
+    TRY(st);
+    ctx->split_ws = ctx->allocs.back();
+    ctx->allocs.pop_back();
+    std::vector<double> w(nrow * np, 0.0);
+    for (int j = 0; j < ctx->p; ++j)
+        w[(size_t)m.sp.orow_h[obs->step[j]] * np + obs->idx[j]] += 1.0 / (obs->sigma[j] * obs->sigma[j]);
+    cudaError_t e = cudaSuccess;
+    if ((e = up(ctx, work, w.data(), w.size())) || (e = cudaStreamSynchronize(ctx->s)))
         return fail(ctx, RIOT_ECUDA, "setup upload failed: %s", cudaGetErrorString(e));
+    m.sp.wgt = work;
+    m.sp.rows = work + nrow * np;
+    m.sp.a = m.sp.rows + cols * nrow * np;
+    m.sp.b = m.sp.a + cols * np;
+    m.sp.cols = (int)cols;
     return RIOT_OK;
 }
 
@@ -636,7 +658,7 @@ riot_status setup_l96(riot_ctx *ctx, const riot_model_desc *model, const riot_ob
     m.band32 = ctx->band32;
     m.sig64 = ctx->sig64;
     m.sig32 = ctx->sig32;
-    TRY(setup_split(ctx, optr, oidx, rinv));
+    TRY(setup_obs_rows(ctx, optr));
     if (ctx->prec == RIOT_PREC_MIXED && warp_kernel_fits(m.geom)) {
         // tables of the warp-synchronous FP32 Hessian kernel
         std::vector<int> ostep, ostart, sslot, perm;
@@ -1421,6 +1443,7 @@ void riot_destroy(riot_ctx *ctx)
     if (ctx->s) cudaStreamSynchronize(ctx->s);
     pc_free(ctx);
     for (const riot_alloc_rec &a : ctx->allocs) ctx_free(ctx, a);
+    ctx_free(ctx, ctx->split_ws);
     for (int i = 0; i < 32; ++i)
         if (ctx->ev[i]) cudaEventDestroy(ctx->ev[i]);
     delete ctx;
@@ -1486,6 +1509,7 @@ riot_status riot_setup(riot_ctx **out, const riot_model_desc *model, const riot_
     }
     for (int i = 0; i < 32; ++i)
         if (cudaEventCreate(&ctx->ev[i]) != cudaSuccess) return bail(fail(ctx, RIOT_ECUDA, "cudaEventCreate failed"));
+    if (model->kind == RIOT_MODEL_L96 && (st = setup_split(ctx, obs)) != RIOT_OK) return bail(st);
     *out = ctx;
     return RIOT_OK;
 }

@@ -60,6 +60,12 @@ struct SplitWork {
     const double *wgt = nullptr;     // [nrow][n] sum of 1/sigma^2 over the observations of a variable
     double *rows = nullptr;          // [cols][nrow][n]
     double *a = nullptr, *b = nullptr;   // [cols][n] states
+    void drop()                          // the workspace (not the tables) is gone
+    {
+        cols = 0;
+        wgt = nullptr;
+        rows = a = b = nullptr;
+    }
 };
 
 struct L96Dev {
