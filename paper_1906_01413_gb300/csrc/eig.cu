@@ -1000,7 +1000,8 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
         int k = jobs[i].k, per_sm = 0;
         const size_t smem = tridiag_smem(k, false);
         const void *fn = (const void *)tridiag_kernel;
-        if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+        static std::atomic<unsigned long long> done{0};
+        if ((err = smem_limit(fn, tridiag_smem(4096, false), done)) != cudaSuccess ||
             (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
             return err;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -1016,7 +1017,8 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
         const size_t smem = tridiag_smem(order[at].k, true);
         const void *fn = (const void *)tridiag_group_kernel;
         int per_sm = 0, ctas = 0;
-        if ((err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
+        static std::atomic<unsigned long long> done{0};
+        if ((err = smem_limit(fn, tridiag_smem(4 * sms, true), done)) != cudaSuccess ||   // the largest resident order
             (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
             return err;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;

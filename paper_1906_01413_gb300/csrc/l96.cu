@@ -418,8 +418,9 @@ cudaError_t bsqrt_launch(const L96Dev &m, const double *in, int64_t ldi, double 
 {
     if (ncols <= 0) return cudaSuccess;
     const int n = m.geom.n;
-    const size_t sm = sizeof(double) * (kBsqrtBlock + m.band.hl + m.band.hh);   // at most 64 + 8191 values
-    cudaError_t e = cudaFuncSetAttribute(bsqrt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const size_t sm = sizeof(double) * (kBsqrtBlock + m.band.hl + m.band.hh);
+    static std::atomic<unsigned long long> done{0};
+    cudaError_t e = smem_limit((const void *)bsqrt_kernel, sizeof(double) * (kBsqrtBlock + 8191), done);   // n = 8192
     if (e != cudaSuccess) return e;
     for (int c0 = 0; c0 < ncols; c0 += 65535) {
         const dim3 grid((n + kBsqrtBlock - 1) / kBsqrtBlock, ncols - c0 < 65535 ? ncols - c0 : 65535);

@@ -32,6 +32,18 @@ int num_sms()
     return sms > 0 ? sms : 1;
 }
 
+cudaError_t smem_limit(const void *kern, size_t bytes, std::atomic<unsigned long long> &done)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ULL << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+
 // ---------------------------------------------------------------------------
 // GEMM: C = alpha op(A) op(B) + beta C, double accumulation.
 // 32 x 32 output tile per CTA, 256 threads, 2 x 2 outputs per thread.
