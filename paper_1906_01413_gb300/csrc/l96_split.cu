@@ -125,6 +125,15 @@ struct LinSteps {
     long long lds, ldr;          // columns of the states, of the rows
 };
 
+// A state's value at place o of its row: times its weight where there are weights, and 0 without an
+// observation whatever the value (an infinity times zero would be NaN).
+__device__ __forceinline__ double row_value(const double *wgt, size_t o, double x)
+{
+    if (!wgt) return x;
+    const double w = wgt[o];
+    return __double_as_longlong(w) == 0 ? 0.0 : w * x;
+}
+
 // Tangent-linear steps t0 .. t1 - 1; the (weighted) state of every observed step goes to its row.
 template <bool RING>
 __global__ void __launch_bounds__(512) tl_steps_kernel(const LinSteps a)
@@ -146,7 +155,7 @@ __global__ void __launch_bounds__(512) tl_steps_kernel(const LinSteps a)
         if (t == max(a.t0, a.t1 - 2)) cudaTriggerProgrammaticLaunchCompletion();
         if (row >= 0 && p.own) {
             const size_t o = (size_t)row * n + p.i;
-            rows[o] = a.wgt ? a.wgt[o] * x : x;
+            rows[o] = row_value(a.wgt, o, x);
         }
         if (t + 1 < a.t1) {
 #pragma unroll
@@ -172,7 +181,7 @@ __global__ void __launch_bounds__(512) tl_steps_kernel(const LinSteps a)
     if (a.last) {
         if (row >= 0) {
             const size_t o = (size_t)row * n + p.i;
-            rows[o] = a.wgt ? a.wgt[o] * x : x;
+            rows[o] = row_value(a.wgt, o, x);
         }
     } else {
         a.out[(size_t)blockIdx.y * a.lds + p.i] = x;
