@@ -709,10 +709,6 @@ template <typename R>
 struct Tab;
 template <>
 struct Tab<float> {
-    static const float *u(const AdvDev &m) { return m.u32; }
-    static const float *v(const AdvDev &m) { return m.v32; }
-    static const float *amp(const AdvDev &m) { return m.amp32; }
-    static const float *kz(const AdvDev &m) { return m.kz32; }
     static const float *w(const AdvDev &m) { return m.w32; }
     static const float *rinv(const AdvDev &m) { return m.rinv32; }
     static const float *Sx(const AdvDev &m) { return m.Sx32; }
@@ -721,10 +717,6 @@ struct Tab<float> {
 };
 template <>
 struct Tab<double> {
-    static const double *u(const AdvDev &m) { return m.u64; }
-    static const double *v(const AdvDev &m) { return m.v64; }
-    static const double *amp(const AdvDev &m) { return m.amp64; }
-    static const double *kz(const AdvDev &m) { return m.kz64; }
     static const double *w(const AdvDev &m) { return m.w64; }
     static const double *rinv(const AdvDev &m) { return m.rinv64; }
     static const double *Sx(const AdvDev &m) { return m.Sx64; }

@@ -785,8 +785,6 @@ riot_status setup_advdiff(riot_ctx *ctx, const riot_model_desc *model, const rio
     const float *rinv32 = nullptr, *w32 = nullptr, *Eb32 = nullptr;
     TRY(upload2(ctx, u, &a.u64, &a.u32));
     TRY(upload2(ctx, v, &a.v64, &a.v32));
-    TRY(upload2(ctx, amp, &a.amp64, &a.amp32));
-    TRY(upload2(ctx, kz, &a.kz64, &a.kz32));
     TRY(upload2(ctx, Sx, &a.Sx64, &a.Sx32));
     TRY(upload2(ctx, Sy, &a.Sy64, &a.Sy32));
     TRY(upload2(ctx, Eb, &a.Eb, &Eb32));

@@ -196,8 +196,8 @@ struct AdvDev {
     const float *w32 = nullptr;
     const double *y = nullptr, *rinv64 = nullptr;
     const float *rinv32 = nullptr;
-    const double *u64 = nullptr, *v64 = nullptr, *amp64 = nullptr, *kz64 = nullptr;
-    const float *u32 = nullptr, *v32 = nullptr, *amp32 = nullptr, *kz32 = nullptr;
+    const double *u64 = nullptr, *v64 = nullptr;
+    const float *u32 = nullptr, *v32 = nullptr;
     const double *Sx64 = nullptr, *Sy64 = nullptr;   // symmetric square roots, row-major
     const float *Sx32 = nullptr, *Sy32 = nullptr;
     const double *Eb = nullptr;       // [n] background emissions
