@@ -752,8 +752,8 @@ cudaError_t step_z_launch(const StepArgsZ &a, int P, cudaStream_t s)
     constexpr int TY = RW * NW - 2 * kHalo;
     const size_t smem = sizeof(pair_t) * (kZRing + 2 * 3) * RW * NW * 32 + sizeof(ulonglong2) * 2 * kZLevels;
     auto kern = adv_step_z_kernel<NW, RW, ADJ, PAIR>;
-    static std::atomic<unsigned long long> done{0};
-    const cudaError_t e = smem_limit((const void *)kern, smem, done);
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.nx + kZTX - 1) / kZTX, (a.ny + TY - 1) / TY, P);
     kern<<<grid, 32 * NW, smem, s>>>(a);
@@ -767,8 +767,8 @@ cudaError_t step_f2_nz(const StepArgsF2 &a, int P, cudaStream_t s)
     constexpr int RX = TX + 2 * kHalo, RY = TY + 2 * kHalo;
     const size_t smem = sizeof(float2) * 2 * (size_t)NZP * RX * RY;
     auto kern = adv_step_f2_kernel<NZP, TX, TY, ADJ>;
-    static std::atomic<unsigned long long> done{0};
-    const cudaError_t e = smem_limit((const void *)kern, smem, done);
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     dim3 grid((a.nx + TX - 1) / TX, (a.ny + TY - 1) / TY, P);
     return launch_after(kern, grid, RX * RY, smem, s, a);

@@ -1000,8 +1000,8 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
         int k = jobs[i].k, per_sm = 0;
         const size_t smem = tridiag_smem(k, false);
         const void *fn = (const void *)tridiag_kernel;
-        static std::atomic<unsigned long long> done{0};
-        if ((err = smem_limit(fn, tridiag_smem(4096, false), done)) != cudaSuccess ||
+        static SmemLimit limit;
+        if ((err = limit.raise(fn, smem)) != cudaSuccess ||
             (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
             return err;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -1017,8 +1017,8 @@ cudaError_t tridiag_run(const TridiagJob *jobs, int njobs, cudaStream_t s)
         const size_t smem = tridiag_smem(order[at].k, true);
         const void *fn = (const void *)tridiag_group_kernel;
         int per_sm = 0, ctas = 0;
-        static std::atomic<unsigned long long> done{0};
-        if ((err = smem_limit(fn, tridiag_smem(4 * sms, true), done)) != cudaSuccess ||   // the largest resident order
+        static SmemLimit limit;
+        if ((err = limit.raise(fn, smem)) != cudaSuccess ||
             (err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, 256, smem)) != cudaSuccess)
             return err;
         if (per_sm < 1) return cudaErrorInvalidConfiguration;
@@ -1080,15 +1080,13 @@ cudaError_t tridiag_finish(int k, double *lam, double *Z, double *work, int *inf
         count_launch();
         if (inviter_smem_bytes(k, 4) <= lim) {
             const size_t sm = inviter_smem_bytes(k, 4);
-            if ((err = cudaFuncSetAttribute(inviter_smem_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sm)) != cudaSuccess)
-                return err;
+            static SmemLimit limit;
+            if ((err = limit.raise((const void *)inviter_smem_kernel<4>, sm)) != cudaSuccess) return err;
             inviter_smem_kernel<4><<<(k + 3) / 4, 128, sm, s>>>(d, e, blo, bhi, k, w, tnorm, Zt, wrq);
         } else if (inviter_smem_bytes(k, 1) <= lim) {
             const size_t sm = inviter_smem_bytes(k, 1);
-            if ((err = cudaFuncSetAttribute(inviter_smem_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sm)) != cudaSuccess)
-                return err;
+            static SmemLimit limit;
+            if ((err = limit.raise((const void *)inviter_smem_kernel<1>, sm)) != cudaSuccess) return err;
             inviter_smem_kernel<1><<<k, 32, sm, s>>>(d, e, blo, bhi, k, w, tnorm, Zt, wrq);
         } else {
             inviter_kernel<<<(k + 3) / 4, 4, 0, s>>>(d, e, blo, bhi, k, w, tnorm, Zt, u0, u1, u2, ml, piv, wrq);

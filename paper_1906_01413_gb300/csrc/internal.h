@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <vector>
 
 #include "../../include/riot.h"
@@ -419,10 +420,17 @@ cudaError_t gather_cols(const double *in, int64_t ldi, const int *perm, int m, i
 cudaError_t fix_col_signs(double *U, int64_t n, int k, int64_t ld, cudaStream_t s);
 
 int num_sms();
-// Lets a kernel take `bytes` of dynamic shared memory on the current device: the most that any call
-// asks for, since the limit is the process's (a call that set its own need could lower it between
-// another host thread's setting and its launch).  done: the devices set so far, one word per kernel.
-cudaError_t smem_limit(const void *kern, size_t bytes, std::atomic<unsigned long long> &done);
+// Dynamic shared memory that a kernel may take, per device.  The limit is the process's: a call that
+// set its own need could lower it between another host thread's setting and its launch, so it is
+// only ever raised.  One static object per kernel.
+class SmemLimit {
+  public:
+    cudaError_t raise(const void *kern, size_t bytes);   // on the current device
+
+  private:
+    std::atomic<size_t> have_[64] = {};
+    std::mutex mu_;
+};
 // host-side count of kernel launches issued by the library
 void count_launch();
 unsigned long long launches_total();

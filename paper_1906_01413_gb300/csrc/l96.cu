@@ -357,25 +357,20 @@ static cudaError_t hvp_launch(const L96Dev &m, const typename V2<real>::type *co
     const int nthr = P * Tp;
     const size_t sm = sizeof(real) * (8 * (size_t)nthr + (size_t)P * stage_pad(m.geom.Np));
     const int grid = (ncols + P - 1) / P;
-    cudaError_t e = cudaSuccess;
+    static SmemLimit limit[3];
+    auto launch = [&](auto kern, SmemLimit &lim) {
+        const cudaError_t e = lim.raise((const void *)kern, sm);
+        if (e != cudaSuccess) return e;
+        count_launch();
+        kern<<<grid, nthr, sm, s>>>(a);
+        return cudaGetLastError();
+    };
     switch (m.geom.E) {
-    case 4:
-        e = cudaFuncSetAttribute(l96_hvp_kernel<real, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_hvp_kernel<real, 4><<<grid, nthr, sm, s>>>(a); }
-        break;
-    case 8:
-        e = cudaFuncSetAttribute(l96_hvp_kernel<real, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_hvp_kernel<real, 8><<<grid, nthr, sm, s>>>(a); }
-        break;
-    case 16:
-        e = cudaFuncSetAttribute(l96_hvp_kernel<real, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) { count_launch(); l96_hvp_kernel<real, 16><<<grid, nthr, sm, s>>>(a); }
-        break;
-    default:
-        return cudaErrorInvalidValue;
+    case 4: return launch(l96_hvp_kernel<real, 4>, limit[0]);
+    case 8: return launch(l96_hvp_kernel<real, 8>, limit[1]);
+    case 16: return launch(l96_hvp_kernel<real, 16>, limit[2]);
+    default: return cudaErrorInvalidValue;
     }
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
 }
 
 cudaError_t l96_hvp_launch_f64(const L96Dev &m, const double2 *coef, const double *W, double *Y, int64_t ld,
@@ -418,9 +413,9 @@ cudaError_t bsqrt_launch(const L96Dev &m, const double *in, int64_t ldi, double 
 {
     if (ncols <= 0) return cudaSuccess;
     const int n = m.geom.n;
-    const size_t sm = sizeof(double) * (kBsqrtBlock + m.band.hl + m.band.hh);
-    static std::atomic<unsigned long long> done{0};
-    cudaError_t e = smem_limit((const void *)bsqrt_kernel, sizeof(double) * (kBsqrtBlock + 8191), done);   // n = 8192
+    const size_t sm = sizeof(double) * (kBsqrtBlock + m.band.hl + m.band.hh);   // at most 64 + 8191 values
+    static SmemLimit limit;
+    cudaError_t e = limit.raise((const void *)bsqrt_kernel, sm);
     if (e != cudaSuccess) return e;
     for (int c0 = 0; c0 < ncols; c0 += 65535) {
         const dim3 grid((n + kBsqrtBlock - 1) / kBsqrtBlock, ncols - c0 < 65535 ? ncols - c0 : 65535);

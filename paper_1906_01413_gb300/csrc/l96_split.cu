@@ -402,7 +402,7 @@ cudaError_t rows_zero(const L96Dev &m, cudaStream_t s)
 cudaError_t l96_nl_launch(const L96Dev &m, const double *x0, double *traj, double2 *coef64, double *xT, cudaStream_t s)
 {
     const int n = m.geom.n, T = m.T;
-    const SplitPlan pl = split_plan(n, 1);
+    const SplitPlan pl = T > 0 ? split_plan(n, 1) : SplitPlan{0, 0, 0.0};
     // A launch's CTAs read the start while others write, so a start that overlaps what is written is
     // set aside (one that is row 0 itself is only written with its own values).  Without a
     // trajectory the states of successive launches alternate between xT and a temporary.

@@ -724,7 +724,8 @@ static cudaError_t launch_tma(const TmaArgs &a, int grid, int nthr, size_t sm, c
 {
     const bool ragged = a.geom.g != 0;
     auto kern = ragged ? l96_hvp_tma_kernel<E, PR, MAXT, true, MINB> : l96_hvp_tma_kernel<E, PR, MAXT, false, MINB>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    static SmemLimit limit[2];
+    const cudaError_t e = limit[ragged].raise((const void *)kern, sm);
     if (e != cudaSuccess) return e;
     count_launch();
     kern<<<grid, nthr, sm, s>>>(a);
@@ -887,9 +888,8 @@ cudaError_t hvp_batch_plan(const HvpBatchWindow *w, int nwin, int P_cap, int S_r
     // a copy from pageable memory may still be in flight when cudaMemcpy returns, and the batch
     // kernel runs on streams that do not wait for the legacy stream: finish it here
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(l96_hvp_batch_kernel<kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)smem)) != cudaSuccess)
-        return e;
+    static SmemLimit limit;
+    if ((e = limit.raise((const void *)l96_hvp_batch_kernel<kThreads>, smem)) != cudaSuccess) return e;
     plan->nwin = nwin;
     plan->nitems = (int)its.size();
     plan->nthr = kThreads;

@@ -647,8 +647,8 @@ size_t warp_smem_bytes(int NW, int S, int slot4, int PR, int Np)
 template <int E, int PR, bool RAGGED, bool SHFL>
 cudaError_t launch_warp(const WarpArgs &a, int grid, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(l96_hvp_warp_kernel<E, PR, RAGGED, SHFL>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit;
+    const cudaError_t e = limit.raise((const void *)l96_hvp_warp_kernel<E, PR, RAGGED, SHFL>, smem);
     if (e != cudaSuccess) return e;
     count_launch();
     l96_hvp_warp_kernel<E, PR, RAGGED, SHFL><<<grid, 32 * a.nwarps, smem, s>>>(a);

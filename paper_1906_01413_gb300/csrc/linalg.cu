@@ -32,15 +32,17 @@ int num_sms()
     return sms > 0 ? sms : 1;
 }
 
-cudaError_t smem_limit(const void *kern, size_t bytes, std::atomic<unsigned long long> &done)
+cudaError_t SmemLimit::raise(const void *kern, size_t bytes)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    const unsigned long long bit = dev < 64 ? 1ULL << dev : 0;
-    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    if (dev >= 64) return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (bytes <= have_[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(mu_);
+    if (bytes <= have_[dev].load(std::memory_order_relaxed)) return cudaSuccess;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    if (e == cudaSuccess) have_[dev].store(bytes, std::memory_order_release);
     return e;
 }
 
@@ -580,7 +582,8 @@ cudaError_t strsm_right_lt_inv(float *X, int m, int k, int64_t ldx, const float 
     const size_t smem = sizeof(float) * ((size_t)k * R + kTrsmRing * 1024);
     if (smem <= 227 * 1024) {
         auto kern = tall ? strsm_lt_rows_kernel<4> : strsm_lt_rows_kernel<1>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        static SmemLimit limit[2];
+        cudaError_t e = limit[tall].raise((const void *)kern, smem);
         if (e != cudaSuccess) return e;
         count_launch();
         kern<<<(m + R - 1) / R, 256, smem, s>>>(X, m, k, ldx, L, ldl);
@@ -1339,7 +1342,8 @@ static cudaError_t dtrsm_rows(double *X, int m, int k, int64_t ldx, const double
 {
     const size_t smem = sizeof(double) * (4 * (size_t)k + 2 * NB * (NB + 1));
     auto kern = lt ? dtrsm_rows_kernel<true> : dtrsm_rows_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static SmemLimit limit[2];
+    cudaError_t e = limit[lt].raise((const void *)kern, smem);
     if (e != cudaSuccess) return e;
     count_launch();
     kern<<<(m + 3) / 4, 128, smem, s>>>(X, m, k, ldx, L, ldl, dinv);

@@ -586,12 +586,8 @@ cudaError_t tc_sgemm(char ta, char tb, int m, int n, int k, float alpha, const f
                      cudaStream_t s)
 {
     if (m <= 0 || n <= 0) return cudaSuccess;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static SmemLimit limit;
+    if (const cudaError_t e = limit.raise((const void *)tc_gemm_kernel, kSmemBytes)) return e;
     const int tiles_m = (m + BM - 1) / BM, tiles_n = (n + BN - 1) / BN;
     int S = (num_sms() + tiles_m * tiles_n - 1) / (tiles_m * tiles_n);
     const int kchunks = (k + BK - 1) / BK;
@@ -647,13 +643,8 @@ cudaError_t tc_gram_f32(int n, int k, const float *Y, int64_t ldy, double *G, in
                         cudaStream_t s)
 {
     if (k <= 0) return cudaSuccess;
-    static bool attr_done = false;
-    if (!attr_done) {
-        cudaError_t e = cudaFuncSetAttribute(tc_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kGramSmemBytes);
-        if (e != cudaSuccess) return e;
-        attr_done = true;
-    }
+    static SmemLimit limit;
+    if (const cudaError_t e = limit.raise((const void *)tc_gram_kernel, kGramSmemBytes)) return e;
     unsigned long long *acc = (unsigned long long *)ws;
     int *colexp = (int *)(acc + (size_t)k * k);
     float2 *colscale = (float2 *)(((uintptr_t)(colexp + k) + 15) & ~(uintptr_t)15);
