@@ -152,9 +152,9 @@ struct Ring {
         if (!aborted) landed = c + 1;
     }
     // Thread 0 only, behind the barrier of stage c: refill the buffer of stage c - 1 with stage
-    // c - 1 + S.  Every thread has used its coefficients of stage c - 1 by then (the values it
-    // published before the barrier depend on the last ones it loaded); those of stage c may
-    // still be on their way to registers.
+    // c - 1 + S.  Every thread has its coefficients of stage c - 1 by then: what it published before
+    // the barrier depends on the neighbours' values of that stage, which it loaded after them, and
+    // a warp's shared loads return in order.  Those of stage c may still be on their way.
     __device__ void refill(int c, int slot)
     {
         if (threadIdx.x == 0 && c > 0 && c - 1 + S < total && !aborted) issue(c - 1 + S, slot ? slot - 1 : S - 1);
@@ -259,6 +259,7 @@ __device__ __forceinline__ void stage_inputs(Coefs<E> &cc, const CoefAt &at, con
     if (!EARLY) {
         ring.wait_ready(sa.c, sa.slot, sa.phase, err);
         load_coefs<E, AD>(cc, ring.slot4(sa.slot), at);
+        asm volatile("" ::: "memory");   // in this order, as refill needs it
     }
 #pragma unroll
     for (int i = 0; i < 3; ++i) get[i] = Hb[i * nthr + from[i]];
