@@ -125,8 +125,8 @@ __global__ void adv_coef_kernel(const double *u, const double *v, int nx, int ny
 // pairs takes 3 cycles of its sub-partition (2 with one of them reused, hence the order of the
 // operations over a warp's rows); the 10 packed operations of a pair and stage make 80 us of the
 // 192 x 192 x 30, 32-column step with the halo's recomputation (64 x 36 regions, 76 % of the rows
-// and 75 % of the columns owned), the shared-memory pipe 55 % of the time.  Measured: 262 -> 182
-// us per step (column form -> this), 32 columns of 240 steps 132.8 -> 90.4 ms, with the same
+// and 75 % of the columns owned), the shared-memory pipe 62 % of the time.  Measured: 262 -> 176
+// us per step (column form -> this, ncu), 32 columns of 240 steps 132.8 -> 89.7 ms, with the same
 // error.  Slower: 16 warps of two rows (97 ms), 8 of four (98 ms), scalar east and west products
 // (mixed with packed ones they stall, 103 ms), barrier before the copies (97 ms).  Coefficients
 // multiplied by a_s beforehand save nothing and round the balance of the vertical fluxes (error
@@ -814,7 +814,7 @@ constexpr int kZWarps = 12, kZRows = 3;   // 64 x 36 regions of 384 threads with
 // FP32 steps.  Both forms take whole waves of one CTA per SM; measured per wave on the 30-level
 // grid 32 us for the level-marching form (0.92 us per level and 1 us) and 8.6 us for the
 // column form (0.47 us per pair of levels and 1.5 us).  192 x 192 x 30, 32 columns: 6 waves,
-// 182 us, against 31 waves, 262 us; one column of it 32 against 9 us.
+// 176 us, against 31 waves, 262 us; one column of it 32 against 9 us.
 cudaError_t step_f32(const AdvDev &m, const float *cin, float *cout, int P, const float *src, long long sstride,
                      float *ebar, long long estride, bool adj, cudaStream_t s)
 {

@@ -151,10 +151,10 @@ cudaError_t conv(const float *in, int ci, const float *W, const float *bias, con
 // share 9 loads.  Slots' sums are then added in FP64.  A sum that is not finite (a product may
 // leave the FP32 range) or so small that the rounding errors of its products may be below that
 // range is formed again in FP64.
-// Bound: FP32 issue (77 % of the slots with unpacked operations, 2.20 ms a training batch; packed
-// 2.07), 16 warps an SM for the loads of 4 positions in flight (24 warps with 2: 2.23 ms).  n = 4096,
-// batch 8, 8 - 64 - 64 - 64 - 128 channels: FP64 sums 12.2 ms, this 1.18 ms, the same gradient error
-// (6.8e-7, that of the FP32 factors).  Fast2Sum without its ordering, 4 operations a term, took
+// Bound: the FP32 pipe (70 to 72 % active; unpacked operations were bound by issue at 77 %, 2.20 ms a
+// training batch against 2.07), 16 warps an SM with the loads of 4 positions in flight (24 warps with
+// 2: 2.23 ms).  n = 4096, batch 8, 8 - 64 - 64 - 64 - 128 channels: FP64 sums 12.2 ms, this 1.13 ms,
+// the same gradient error (6.8e-7, that of the FP32 factors).  Fast2Sum without its ordering, 4 operations a term, took
 // 0.93 ms and was off by 6 % where a lane's terms cancel to 2^-21.
 constexpr int kGradO = 4;
 
